@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "blockfact.h"
+#include "densetail.h"
 #include "internal.h"
 
 namespace exago {
@@ -412,6 +413,97 @@ __global__ void __launch_bounds__(kNT) k_bf_backward(const DevSymK S, int B, con
     for (int i = 0; i < BS; i++) x[((size_t)J * BS + i) * B + b] = v[i];
 }
 
+// The tail's panels from the assembled blocks: T_IJ = A_IJ - sum over the columns K < k0 of
+// F_IK U_KJ, one thread per (state, lower block of the tail), written where densetail.h keeps it
+// (LU: the upper block, transposed, into V; inside a 64-column panel's own square also in place).
+template <int BS, bool SYM>
+__global__ void __launch_bounds__(kNT) k_bf_tail(const DevSymK S, int B, const double *T,
+                                                 const double *TU, const double *L,
+                                                 const double *U, double *D, double *V,
+                                                 size_t dstride) {
+    constexpr int BB = BS * BS;
+    const int b = blockIdx.y * kNT + threadIdx.x;
+    if (b >= B) return;
+    const int e = blockIdx.x;
+    int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);   // e = i (i + 1) / 2 + j
+    while (i * (i + 1) / 2 > e) i--;
+    while ((i + 1) * (i + 2) / 2 <= e) i++;
+    const int j = e - i * (i + 1) / 2;
+    double acc[BB], accU[BB];
+#pragma unroll
+    for (int k = 0; k < BB; k++) { acc[k] = 0.0; accU[k] = 0.0; }
+    const int t = __ldg(S.tail_tgt + e);
+    if (t >= 0) {
+        const int p = __ldg(S.tgt_blk + t);
+        load_blk_cg<BS>(T, p, B, b, acc);
+        if (!SYM) load_blk_cg<BS>(TU, p, B, b, accU);
+        for (int64_t q = __ldg(S.tptr + t), q1 = __ldg(S.tail_q1 + t); q < q1; q++) {
+            const int2 pr = __ldg(S.pairs + q);
+            if (!EXAGO_DCHECK(S, pr.x >= 0 && pr.x < S.nblk && pr.y >= 0 && pr.y < S.nblk)) continue;
+            double X[BB], Y[BB];
+            load_blk_cg<BS>(T, pr.x, B, b, X);
+            load_blk_cg<BS>(SYM ? L : U, pr.y, B, b, Y);
+            sub_mul<BS, SYM>(acc, X, Y);
+            if (!SYM && i != j) {
+                load_blk_cg<BS>(T, pr.y, B, b, X);
+                load_blk_cg<BS>(U, pr.x, B, b, Y);
+                sub_mul<BS, false>(accU, X, Y);
+            }
+        }
+    }
+    const int n = S.tail_n, r0 = BS * i, c0 = BS * j;
+    double *Db = D + (size_t)b * dstride, *Vb = SYM ? nullptr : V + (size_t)b * dstride;
+#pragma unroll
+    for (int c = 0; c < BS; c++)
+#pragma unroll
+        for (int r = 0; r < BS; r++) {
+            Db[tail_pos(n, r0 + r, c0 + c)] = acc[r * BS + c];
+            if (SYM || i == j) continue;
+            if ((r0 >> 6) == (c0 >> 6)) Db[tail_pos(n, c0 + c, r0 + r)] = accU[c * BS + r];
+            else Vb[tail_pos(n, r0 + r, c0 + c)] = accU[c * BS + r];
+        }
+}
+
+// Identity in the rows that pad the tail to a multiple of 64: one thread per entry and state.
+__global__ void __launch_bounds__(kNT) k_bf_tail_pad(int n, int nreal, double *D, double *V,
+                                                     size_t dstride) {
+    const int e = blockIdx.x * kNT + threadIdx.x;
+    if (e >= (n - nreal) * n) return;
+    const int row = nreal + e % (n - nreal), col = e / (n - nreal);
+    const size_t b = blockIdx.y;
+    if (row >= (col & ~63)) {
+        D[b * dstride + tail_pos(n, row, col)] = row == col ? 1.0 : 0.0;
+        if (V) V[b * dstride + tail_pos(n, row, col)] = 0.0;
+    }
+    // LU: the padding columns of a panel's own square, above the padding rows
+    if (V && (row >> 6) == (col >> 6) && col < nreal) D[b * dstride + tail_pos(n, col, row)] = 0.0;
+}
+
+// Right-hand side of the tail: r_J - sum over K < k0 of F_JK z_K, one thread per (state, column).
+template <int BS>
+__global__ void __launch_bounds__(kNT) k_bf_tail_rhs(const DevSymK S, int B, const double *T, double *x) {
+    const int b = blockIdx.y * kNT + threadIdx.x;
+    if (b >= B) return;
+    const int J = S.k0 + blockIdx.x;
+    double y[BS];
+#pragma unroll
+    for (int i = 0; i < BS; i++) y[i] = __ldcg(x + ((size_t)J * BS + i) * B + b);
+    for (int64_t r = __ldg(S.rowptr + J), r1 = __ldg(S.tail_r1 + J); r < r1; r++) {
+        const int K = __ldg(S.rowcol + r), p = __ldg(S.rowblk + r);
+        if (!EXAGO_DCHECK(S, K >= 0 && K < S.nb && p >= 0 && p < S.nblk)) continue;
+        double F[BS * BS], z[BS];
+        load_blk<BS>(T, p, B, b, F);
+#pragma unroll
+        for (int i = 0; i < BS; i++) z[i] = __ldcg(x + ((size_t)K * BS + i) * B + b);
+#pragma unroll
+        for (int i = 0; i < BS; i++)
+#pragma unroll
+            for (int k = 0; k < BS; k++) y[i] = fma(-F[i * BS + k], z[k], y[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < BS; i++) x[((size_t)J * BS + i) * B + b] = y[i];
+}
+
 }  // namespace
 
 // A level is split when it has fewer than this many targets (factor) or columns (sweeps): a
@@ -420,11 +512,11 @@ constexpr int kSplitBelow = 64;
 
 template <int BS, bool SYM>
 int launch_block_factor(const DevSym &S, int B, double *T, double *TU, double *L, double *U,
-                        int *neg, int *bad, double tiny, cudaStream_t st) {
+                        int *neg, int *bad, double tiny, void *tail, cudaStream_t st) {
     if (B <= 0) return 0;
     const unsigned gy = (unsigned)((B + kNT - 1) / kNT), gy32 = (unsigned)((B + 31) / 32);
     for (int l = 0; l < S.nlevels; l++) {
-        const int t0 = S.lvl_tptr[l], nt = S.lvl_tptr[l + 1] - t0;
+        const int t0 = S.lvl_tptr[l], nt = S.sp_tgts[l];
         if (nt <= 0) continue;
         const dim3 grid((unsigned)nt, gy);
         if (nt < kSplitBelow)
@@ -434,16 +526,31 @@ int launch_block_factor(const DevSym &S, int B, double *T, double *TU, double *L
             k_bf_update<BS, SYM><<<grid, kNT, 0, st>>>(S.k, B, T, TU, L, U, t0);
         k_bf_scale<BS, SYM><<<grid, kNT, 0, st>>>(S.k, B, T, TU, L, U, neg, bad, tiny, t0);
     }
+    if (S.k.tail_n > 0) {
+        const int n = S.k.tail_n, R = S.k.nb - S.k.k0, nreal = R * BS;
+        const TailShape ts = tail_shape(n, B, SYM);
+        double *D = (double *)((char *)tail + ts.dn);
+        double *V = SYM ? nullptr : (double *)((char *)tail + ts.dv);
+        k_bf_tail<BS, SYM><<<dim3((unsigned)(R * (R + 1) / 2), gy), kNT, 0, st>>>(
+            S.k, B, T, TU, L, U, D, V, ts.dense_doubles);
+        for (int b0 = 0; n > nreal && b0 < B; b0 += 65535)
+            k_bf_tail_pad<<<dim3((unsigned)(((n - nreal) * n + kNT - 1) / kNT),
+                                 (unsigned)(B - b0 < 65535 ? B - b0 : 65535)), kNT, 0, st>>>(
+                n, nreal, D + b0 * ts.dense_doubles, V ? V + b0 * ts.dense_doubles : nullptr,
+                ts.dense_doubles);
+        const int e = launch_tail_factor(ts, B, BS, SYM, tail, neg, bad, tiny, S.k.status, st);
+        if (e != 0) return e;
+    }
     return (int)cudaGetLastError();
 }
 
 template <int BS, bool SYM>
 int launch_block_solve(const DevSym &S, int B, const double *T, const double *L, const double *U,
-                       double *x, cudaStream_t st) {
+                       double *x, const void *tail, cudaStream_t st) {
     if (B <= 0) return 0;
     const unsigned gy = (unsigned)((B + kNT - 1) / kNT), gy32 = (unsigned)((B + 31) / 32);
     for (int l = 0; l < S.nlevels; l++) {
-        const int c0 = S.lvl_colptr[l], nc = S.lvl_colptr[l + 1] - c0;
+        const int c0 = S.lvl_colptr[l], nc = S.sp_cols[l];
         if (nc <= 0) continue;
         if (nc < kSplitBelow)
             k_bf_forward_split<BS><<<dim3((unsigned)nc, gy32), 32 * kSweepSlices, 0, st>>>(
@@ -451,8 +558,15 @@ int launch_block_solve(const DevSym &S, int B, const double *T, const double *L,
         else
             k_bf_forward<BS><<<dim3((unsigned)nc, gy), kNT, 0, st>>>(S.k, B, T, L, x, c0);
     }
+    if (S.k.tail_n > 0) {
+        const int R = S.k.nb - S.k.k0;
+        k_bf_tail_rhs<BS><<<dim3((unsigned)R, gy), kNT, 0, st>>>(S.k, B, T, x);
+        const int e = launch_tail_solve(tail_shape(S.k.tail_n, B, SYM), B, R * BS, SYM, tail,
+                                        x + (size_t)S.k.k0 * BS * B, st);
+        if (e != 0) return e;
+    }
     for (int l = S.nlevels - 1; l >= 0; l--) {
-        const int c0 = S.lvl_colptr[l], nc = S.lvl_colptr[l + 1] - c0;
+        const int c0 = S.lvl_colptr[l], nc = S.sp_cols[l];
         if (nc <= 0) continue;
         if (nc < kSplitBelow)
             k_bf_backward_split<BS, SYM><<<dim3((unsigned)nc, gy32), 32 * kSweepSlices, 0, st>>>(
@@ -472,6 +586,11 @@ int upload_block_sym(const BlockSym &S, DevSym &D, std::vector<void *> &allocs) 
     D.k.npairs = (int64_t)S.pairs.size();
     D.lvl_colptr = S.lvl_colptr;
     D.lvl_tptr = S.lvl_tptr;
+    D.sp_cols = S.sp_cols;
+    D.sp_tgts = S.sp_tgts;
+    D.sparse_blocks = S.colptr[S.k0];
+    D.k.k0 = S.k0;
+    D.k.tail_n = S.tail_n;
     auto up = [&](const void *src, size_t bytes, const void **dst) -> int {
         *dst = nullptr;
         if (bytes == 0) return 0;
@@ -483,23 +602,24 @@ int upload_block_sym(const BlockSym &S, DevSym &D, std::vector<void *> &allocs) 
         *dst = p;
         return (int)e;
     };
-    int e = 0;
+    int e = S.tail_n > 0 ? tail_allow_smem() : 0;
 #define UPV(field, vec) \
     if (!e) e = up(S.vec.data(), S.vec.size() * sizeof(S.vec[0]), (const void **)&D.k.field)
     UPV(colptr, colptr); UPV(rowidx, rowidx); UPV(rowptr, rowptr); UPV(rowblk, rowblk);
     UPV(rowcol, rowcol); UPV(lvl_cols, lvl_cols); UPV(tgt_blk, tgt_blk); UPV(tgt_diag, tgt_diag);
-    UPV(tptr, tptr); UPV(pairs, pairs);
+    UPV(tptr, tptr); UPV(pairs, pairs); UPV(tail_tgt, tail_tgt); UPV(tail_q1, tail_q1);
+    UPV(tail_r1, tail_r1);
 #undef UPV
     return e;
 }
 
 template int launch_block_factor<4, true>(const DevSym &, int, double *, double *, double *,
-                                          double *, int *, int *, double, cudaStream_t);
+                                          double *, int *, int *, double, void *, cudaStream_t);
 template int launch_block_factor<2, false>(const DevSym &, int, double *, double *, double *,
-                                           double *, int *, int *, double, cudaStream_t);
+                                           double *, int *, int *, double, void *, cudaStream_t);
 template int launch_block_solve<4, true>(const DevSym &, int, const double *, const double *,
-                                         const double *, double *, cudaStream_t);
+                                         const double *, double *, const void *, cudaStream_t);
 template int launch_block_solve<2, false>(const DevSym &, int, const double *, const double *,
-                                          const double *, double *, cudaStream_t);
+                                          const double *, double *, const void *, cudaStream_t);
 
 }  // namespace exago

@@ -53,6 +53,14 @@ struct BlockSym {
     std::vector<int> tgt_diag;       // block position of the target column's diagonal
     std::vector<int64_t> tptr;       // [ntargets + 1]
     std::vector<int2> pairs;         // (position of (I, K), position of (J, K))
+    // dense tail (densetail.h): the columns k0 .. nb - 1 are factored as one dense matrix per
+    // state (k0 = nb: none).  sp_cols / sp_tgts [nlevels]: columns and targets of each level
+    // below k0 (they come first in the level's lists); tail_q1 [ntargets]: end of each target's
+    // pairs with K < k0; tail_r1 [nb]: end of each row's blocks with K < k0; tail_tgt: the target
+    // of each lower block (I, J) of the tail, row after row, or -1 where the factor has none.
+    int k0 = 0, tail_n = 0;          // first tail column; padded scalar size
+    std::vector<int> sp_cols, sp_tgts, tail_tgt;
+    std::vector<int64_t> tail_q1, tail_r1;
     // solve schedule: for each column, in the level order of lvl_cols
     double flops_factor_per_block = 0;   // sum over pairs of one block product (BS^3 FMA units)
 };
@@ -61,6 +69,10 @@ struct BlockSym {
 // adj [..]; duplicates and self loops are ignored).  Returns false with a message on an
 // inconsistent graph.
 bool build_block_sym(int nb, const int *adj_ptr, const int *adj, BlockSym &S, std::string &err);
+
+// Chooses the dense tail of a factorisation of BS x BS blocks (symmetric or not) from the structure
+// alone, so that a state's factorisation is the same in every batch.
+void choose_tail(BlockSym &S, int BS, bool sym);
 
 // Device tables of a symbolic factorisation (handed to the kernels by value).
 struct DevSymK {
@@ -75,13 +87,17 @@ struct DevSymK {
     const int64_t *tptr;
     const int2 *pairs;
     int *status;             // the owning net's device status word (debug-build index checks)
+    int k0, tail_n;          // dense tail: first column, padded scalar size (0: none)
+    const int *tail_tgt;     // [R (R + 1) / 2]
+    const int64_t *tail_q1, *tail_r1;
 };
 
 // The device tables and the host copies of the launch ranges.
 struct DevSym {
     DevSymK k{};
     int nlevels = 0;
-    std::vector<int> lvl_colptr, lvl_tptr;
+    std::vector<int> lvl_colptr, lvl_tptr, sp_cols, sp_tgts;
+    int64_t sparse_blocks = 0;   // factor blocks of the columns before the tail
 };
 
 // Uploads S (cudaMalloc through dev_malloc; the pointers go to `allocs` for the owner to free).
@@ -89,16 +105,17 @@ int upload_block_sym(const BlockSym &S, DevSym &D, std::vector<void *> &allocs);
 
 // Batched numeric factorisation and solve on DevSym.  T: the assembled matrix A, lower blocks
 // (and TU the upper blocks, the transposed positions, for LU), [nblk][BS*BS][B]; overwritten by
-// F = L D (and U D).  L: [nblk][BS*BS][B] receives L (off-diagonal) and D^-1 (diagonal
-// positions); U likewise for LU.  neg [B] counts the negative pivots of the diagonal blocks'
+// F = L D (and U D) in the columns before the tail.  L: [sparse_blocks][BS*BS][B] receives L
+// (off-diagonal) and D^-1 (diagonal positions) of those columns; U likewise for LU.  tail: the
+// workspace of tail_shape(S.k.tail_n, B, SYM), which receives the tail's factor.  neg [B] counts the negative pivots of the diagonal blocks'
 // in-block elimination (SYM), bad [B] the pivots with |d| below tiny * the block's largest entry.
 template <int BS, bool SYM>
 int launch_block_factor(const DevSym &S, int B, double *T, double *TU, double *L, double *U,
-                        int *neg, int *bad, double tiny, cudaStream_t st);
+                        int *neg, int *bad, double tiny, void *tail, cudaStream_t st);
 // x [nb][BS][B] (elimination index order): on entry the right-hand side, on return the solution.
 // T, L, U as the factorisation left them.
 template <int BS, bool SYM>
 int launch_block_solve(const DevSym &S, int B, const double *T, const double *L, const double *U,
-                       double *x, cudaStream_t st);
+                       double *x, const void *tail, cudaStream_t st);
 
 }  // namespace exago

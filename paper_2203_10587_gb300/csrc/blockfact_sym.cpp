@@ -179,7 +179,80 @@ bool build_block_sym(int nb, const int *adj_ptr, const int *adj, BlockSym &S, st
         });
     }
     S.flops_factor_per_block = (double)S.pairs.size();
+    S.k0 = nb;
+    S.sp_cols.resize(S.nlevels);
+    S.sp_tgts.resize(S.nlevels);
+    for (int l = 0; l < S.nlevels; l++) {
+        S.sp_cols[l] = S.lvl_colptr[l + 1] - S.lvl_colptr[l];
+        S.sp_tgts[l] = S.lvl_tptr[l + 1] - S.lvl_tptr[l];
+    }
     return true;
+}
+
+// The tail that costs least, by what the parts took on GB300 with 128 states: a level of the
+// sparse part 20 us (its launches), a thousand of its 4 x 4 block products 16 us (2 x 2: 4 us),
+// a panel of 64 columns 60 us (its launches and 64 dependent pivots), a dense 64 x 64 x 64 tile
+// product 3.5 us.
+void choose_tail(BlockSym &S, int BS, bool sym) {
+    const int nb = S.nb, step = 64 / BS;
+    std::vector<double> pairs(nb + 1, 0.0);   // block products whose inner column is below k
+    std::vector<int> levels(nb + 1, 0);
+    for (int k = 0; k < nb; k++) {
+        const double d = (double)(S.colptr[k + 1] - S.colptr[k] - 1);
+        pairs[k + 1] = pairs[k] + d * (d + 1) / 2;
+        levels[k + 1] = std::max(levels[k], S.level[k] + 1);
+    }
+    const double side = sym ? 1.0 : 2.0, pair = (BS == 4 ? 0.016 : 0.004) * side;
+    auto sparse = [&](int k0) { return 20.0 * levels[k0] + pair * pairs[k0]; };
+    double best = sparse(nb);
+    int best_k0 = nb, best_n = 0;
+    for (int P = 1;; P++) {   // at most 384 panels: the sweeps hold a state's vector in shared memory
+        const int R = std::min(nb, P * step);
+        const double dense = P * (P + 1.0) * (P + 2.0) / 6.0 * side;
+        const double cost = sparse(nb - R) + 60.0 * P + 3.5 * dense;
+        if (cost < best) {
+            best = cost;
+            best_k0 = nb - R;
+            best_n = 64 * P;
+        }
+        if (R == nb || P == 384 || 60.0 * P + 3.5 * dense > best) break;
+    }
+    if (best_n == 0) return;
+    const int k0 = best_k0, R = nb - k0;
+    S.k0 = k0;
+    S.tail_n = best_n;
+    for (int l = 0; l < S.nlevels; l++) {
+        S.sp_cols[l] = S.sp_tgts[l] = 0;
+        for (int c = S.lvl_colptr[l]; c < S.lvl_colptr[l + 1]; c++) {
+            const int k = S.lvl_cols[c];
+            if (k >= k0) continue;   // ascending within a level: the columns below k0 come first
+            S.sp_cols[l]++;
+            S.sp_tgts[l] += (int)(S.colptr[k + 1] - S.colptr[k]);
+        }
+    }
+    std::vector<int> col_of_blk(S.nblk);
+    for (int k = 0; k < nb; k++)
+        for (int64_t p = S.colptr[k]; p < S.colptr[k + 1]; p++) col_of_blk[p] = k;
+    const int64_t ntgt = (int64_t)S.tgt_blk.size();
+    S.tail_q1.resize(ntgt);
+    S.tail_tgt.assign((size_t)R * (R + 1) / 2, -1);
+    for (int64_t t = 0; t < ntgt; t++) {
+        const int p = S.tgt_blk[t], J = col_of_blk[p];
+        int64_t q = S.tptr[t + 1];
+        if (J >= k0) {   // pairs ascend in K
+            q = S.tptr[t];
+            while (q < S.tptr[t + 1] && col_of_blk[S.pairs[q].y] < k0) q++;
+            const int64_t i = S.rowidx[p] - k0, j = J - k0;
+            S.tail_tgt[(size_t)(i * (i + 1) / 2 + j)] = (int)t;
+        }
+        S.tail_q1[t] = q;
+    }
+    S.tail_r1.resize(nb);
+    for (int i = 0; i < nb; i++) {
+        int64_t r = S.rowptr[i];
+        while (r < S.rowptr[i + 1] && S.rowcol[r] < k0) r++;
+        S.tail_r1[i] = r;
+    }
 }
 
 }  // namespace exago

@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "blockfact.h"
+#include "densetail.h"
 #include "internal.h"
 
 namespace exago {
@@ -254,9 +255,10 @@ struct exago_kkt {
 namespace {
 
 size_t kkt_ws_bytes(const exago_kkt *k, int B) {
-    const size_t blk = (size_t)k->S.nblk * 16 * (size_t)B * sizeof(double);
-    return 2 * round256(blk) + round256((size_t)k->S.nb * 4 * B * sizeof(double)) +
-           round256(2 * (size_t)B * sizeof(int));
+    const size_t entry = 16 * (size_t)B * sizeof(double);
+    return round256((size_t)k->S.nblk * entry) + round256((size_t)k->D.sparse_blocks * entry) +
+           round256((size_t)k->S.nb * 4 * B * sizeof(double)) + round256(2 * (size_t)B * sizeof(int)) +
+           tail_shape(k->S.tail_n, B, true).bytes;
 }
 
 template <typename T>
@@ -324,6 +326,8 @@ exago_status exago_kkt_create(exago_net_t net, exago_kkt_t *out) {
             delete k;
             return set_last_error(EXAGO_EINVAL, "KKT symbolic factorisation: " + err);
         }
+        choose_tail(k->S, 4, true);
+        k->D.sparse_blocks = k->S.colptr[k->S.k0];
         const BlockSym &S = k->S;
         // variable / row index of entry a (0..3) of bus u: Va, Vm (x) or lamP, lamQ (rows)
         auto var = [&](int u, int a) { return a == 0 ? u : a == 1 ? nb + u : a == 2 ? u : nb + u; };
@@ -502,9 +506,11 @@ exago_status exago_kkt_solve(exago_kkt_t kkt, int B, const double *jval, const d
     const size_t blk = round256((size_t)kkt->S.nblk * 16 * (size_t)B * sizeof(double));
     double *T = (double *)w;
     double *L = (double *)(w + blk);
-    double *x = (double *)(w + 2 * blk);
-    int *neg = (int *)(w + 2 * blk + round256((size_t)kkt->S.nb * 4 * B * sizeof(double)));
-    int *bad = neg + B;
+    char *p = w + blk + round256((size_t)kkt->D.sparse_blocks * 16 * (size_t)B * sizeof(double));
+    double *x = (double *)p;
+    p += round256((size_t)kkt->S.nb * 4 * B * sizeof(double));
+    int *neg = (int *)p, *bad = neg + B;
+    void *tail = p + round256(2 * (size_t)B * sizeof(int));
     const KktDev &K = kkt->K;
     const unsigned gy = (unsigned)((B + KNT - 1) / KNT);
     cudaError_t e = cudaMemsetAsync(neg, 0, 2 * (size_t)B * sizeof(int), st);
@@ -512,8 +518,8 @@ exago_status exago_kkt_solve(exago_kkt_t kkt, int B, const double *jval, const d
     k_kkt_assemble<<<dim3((unsigned)kkt->S.nblk, gy), KNT, 0, st>>>(K, kkt->D.k, B, jval, hval, dx,
                                                                     dc, T);
     k_kkt_rhs<<<dim3((unsigned)K.nb, gy), KNT, 0, st>>>(K, B, jval, hval, dx, dc, rhs, x, neg);
-    int le = launch_block_factor<4, true>(kkt->D, B, T, nullptr, L, nullptr, neg, bad, kTiny, st);
-    if (le == 0) le = launch_block_solve<4, true>(kkt->D, B, T, L, nullptr, x, st);
+    int le = launch_block_factor<4, true>(kkt->D, B, T, nullptr, L, nullptr, neg, bad, kTiny, tail, st);
+    if (le == 0) le = launch_block_solve<4, true>(kkt->D, B, T, L, nullptr, x, tail, st);
     if (le == 0) {
         k_kkt_recover_bus<<<dim3((unsigned)K.nb, gy), KNT, 0, st>>>(K, B, jval, hval, dx, rhs, x, sol);
         if (K.nl > 0)

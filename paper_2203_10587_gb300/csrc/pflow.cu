@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "blockfact.h"
+#include "densetail.h"
 #include "internal.h"
 
 namespace exago {
@@ -113,7 +114,7 @@ struct exago_pf {
 namespace {
 
 struct PfLayout {
-    size_t gh, jv, blk, x, cnt, total;
+    size_t gh, jv, blk, sblk, x, cnt, total;   // sblk: the columns before the dense tail
 };
 
 PfLayout pf_layout(const exago_pf *pf, int B) {
@@ -121,9 +122,11 @@ PfLayout pf_layout(const exago_pf *pf, int B) {
     L.gh = r256((size_t)B * pf->P.m * sizeof(double));
     L.jv = r256((size_t)B * pf->P.nnzJ * sizeof(double));
     L.blk = r256((size_t)pf->S.nblk * 4 * B * sizeof(double));
+    L.sblk = r256((size_t)pf->D.sparse_blocks * 4 * B * sizeof(double));
     L.x = r256((size_t)pf->S.nb * 2 * B * sizeof(double));
     L.cnt = r256((size_t)B * (2 * sizeof(int) + sizeof(unsigned long long)));
-    L.total = L.gh + L.jv + 4 * L.blk + L.x + L.cnt;
+    L.total = L.gh + L.jv + 2 * L.blk + 2 * L.sblk + L.x + L.cnt +
+              tail_shape(pf->S.tail_n, B, false).bytes;
     return L;
 }
 
@@ -197,6 +200,7 @@ exago_status exago_pf_create(exago_net_t net, const int *bus_type, exago_pf_t *o
             delete pf;
             return set_last_error(EXAGO_EINVAL, "power-flow symbolic factorisation: " + err);
         }
+        choose_tail(pf->S, 2, false);
         const BlockSym &S = pf->S;
         auto row_active = [&](int u, int a) { return a == 0 ? bus_type[u] != 3 : bus_type[u] == 1; };
         // source of entry (equation a of bus u, unknown c of bus v)
@@ -297,10 +301,13 @@ exago_status exago_pf_step(exago_pf_t pf, const exago_batch *batch, double *x_ne
     double *jv = (double *)(w + Lw.gh);
     char *fw = w + Lw.gh + Lw.jv;
     double *T = (double *)fw, *TU = (double *)(fw + Lw.blk);
-    double *L = (double *)(fw + 2 * Lw.blk), *U = (double *)(fw + 3 * Lw.blk);
-    double *x = (double *)(fw + 4 * Lw.blk);
-    int *neg = (int *)(fw + 4 * Lw.blk + Lw.x);
+    fw += 2 * Lw.blk;
+    double *L = (double *)fw, *U = (double *)(fw + Lw.sblk);
+    fw += 2 * Lw.sblk;
+    double *x = (double *)fw;
+    int *neg = (int *)(fw + Lw.x);
     int *bad = neg + B;
+    void *tail = fw + Lw.x + Lw.cnt;
     unsigned long long *mis = (unsigned long long *)(bad + B);
     // g and J at x (the evaluation of the batch's states; its own scratch is the net's)
     exago_batch eb = *batch;
@@ -315,8 +322,8 @@ exago_status exago_pf_step(exago_pf_t pf, const exago_batch *batch, double *x_ne
     const unsigned gy = (unsigned)((B + PNT - 1) / PNT);
     k_pf_assemble<<<dim3((unsigned)pf->S.nblk, gy), PNT, 0, st>>>(D, B, pf->S.nblk, jv, T, TU);
     k_pf_rhs<<<dim3((unsigned)D.nb, gy), PNT, 0, st>>>(D, B, gh, x, mis);
-    int le = launch_block_factor<2, false>(pf->D, B, T, TU, L, U, neg, bad, kPfTiny, st);
-    if (le == 0) le = launch_block_solve<2, false>(pf->D, B, T, L, U, x, st);
+    int le = launch_block_factor<2, false>(pf->D, B, T, TU, L, U, neg, bad, kPfTiny, tail, st);
+    if (le == 0) le = launch_block_solve<2, false>(pf->D, B, T, L, U, x, tail, st);
     if (le == 0) {
         k_pf_update<<<dim3((unsigned)D.n, gy), PNT, 0, st>>>(D, B, batch->x, x, x_new);
         if (mismatch) k_pf_mismatch<<<(B + 255) / 256, 256, 0, st>>>(mis, mismatch, B);
