@@ -425,7 +425,11 @@ exago_status exago_eval_profile(exago_net_t net, const exago_batch *batch, doubl
 /*
  * Launch configuration of a net (zero-initialised = automatic).
  *   schedule  EXAGO_SCHED_AUTO: the autotuned choice for the batch size if exago_net_autotune ran
- *             for it, else the persistent schedule.  EXAGO_SCHED_KERNELS: one launch per stage
+ *             for it, else the persistent schedule, or, when no field of the configuration is set
+ *             and the grid is small (up to 1,280 branches, by an estimate from the branches and
+ *             the states), one block per state, whose records stay in its shared memory (the
+ *             results are the same bit for bit; exago_net_get_config then still returns the
+ *             persistent settings, which apply once a field is set).  EXAGO_SCHED_KERNELS: one launch per stage
  *             (branch, bus, fixup, gradient, objective) over the batch.  EXAGO_SCHED_PERSISTENT:
  *             one fused launch whose CTAs claim branch and bus tiles of all states from a work
  *             list (the batched evaluation of SCOPFLOW / SOPFLOW subproblems, Sec. V-A, VI-A).

@@ -237,6 +237,7 @@ exago_status do_upload(exago_net *net) {
             if (le2 == 0) le2 = bus_allow_stage();
             if (le2 == 0) le2 = cart_allow_stage();
             if (le2 == 0) le2 = persist_w_allow_stage();
+            if (le2 == 0) le2 = state_allow_smem();
             if (le2 != 0) return cuda_fail((cudaError_t)le2, "cudaFuncSetAttribute");
             done[net->device] = true;
         }
@@ -450,6 +451,51 @@ Resolved resolve(exago_net *net, int B) {
     return r;
 }
 
+// Whether an untouched configuration runs a block per state, and how: threads per block and shared
+// memory (the records, and the rows of the largest bus tile where they fit beside them).
+struct StateBlock {
+    int nt = 0;   // 0: not this schedule
+    int cap = 0;
+    size_t smem = 0;
+};
+
+StateBlock state_block(const exago_net *net, int B) {
+    StateBlock s;
+    const exago_config &c = net->cfg;
+    if (c.schedule != EXAGO_SCHED_AUTO || c.block || c.occupancy || c.stage_records || c.lag ||
+        c.ring || c.chunk || c.use_graph || c.spin_limit || c.test_force_timeout ||
+        c.tile_group || c.tiling || net->tuned.count(B))
+        return s;
+    const size_t rec = (size_t)NCOMP * net->dev.nslot * sizeof(double);
+    if (rec > (size_t)kStateMaxBytes || net->plan.nl > 1280) return s;
+    auto smem_of = [&](int nt, int *cap) {
+        const int rows = net->dev.stage_cap_rows[stage_index(nt)];
+        *cap = rec + rows * sizeof(double) <= (size_t)kStateMaxBytes ? rows : 0;
+        return rec + *cap * sizeof(double);
+    };
+    // Estimated times (us), fitted to 9 grids of 30 to 900 buses x 1 to 1,024 states (all outputs):
+    //   persistent            24 + 0.34 per 1,000 branch items;
+    //   256 threads a state   12 + 0.052 a branch for one block an SM; two resident blocks of a
+    //                         further wave take 0.72 of one's time each;
+    //   64 threads a state    7.5 + 0.14 a branch, the blocks of an SM overlapping (up to 160
+    //                         branches: one pass of 64 threads takes three items each).
+    // For example 118 x 1,024: 77, 100 and 60 (measured 70, 73 and 68); 300 x 304: 64, 46 (68,
+    // 47); 900 x 304: 145, 146 (129, 143).
+    const double nl = net->plan.nl, per_sm = (double)B / (net->sm_count > 0 ? net->sm_count : 1);
+    int cap64, cap256;
+    const size_t b64 = smem_of(64, &cap64), b256 = smem_of(256, &cap256);
+    const bool two = 2 * (b256 + 3072) <= (size_t)net->smem_per_sm;   // with the static part
+    const double waves = std::ceil(per_sm);
+    const double pers = 24.0 + 0.34e-3 * nl * B;
+    const double t256 = (12.0 + 0.052 * nl) * (waves <= 1.0 ? 1.0 : two ? 0.72 * waves : waves);
+    const double t64 = nl > 160 ? 1e30 : (7.5 + 0.14 * nl) * std::max(1.0, 0.6 + 0.22 * per_sm);
+    if (std::min(t64, t256) >= pers) return s;
+    s.nt = t64 < t256 ? 64 : 256;
+    s.cap = t64 < t256 ? cap64 : cap256;
+    s.smem = t64 < t256 ? b64 : b256;
+    return s;
+}
+
 size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
 // Branch-end records of one state.
@@ -661,6 +707,17 @@ exago_status eval_locked(exago_net *net, const exago_batch *bt, double *f, doubl
                          double *gh, double *jval, double *hval, ProfileHook *hook,
                          bool allow_graph, const StateTab *tab, const Resolved &rs, void *ws);
 
+EvalReq request(const exago_batch *bt, double *f, double *grad, double *gh, double *jval,
+                double *hval, const StateTab *tab) {
+    EvalReq R{};
+    R.B = bt->B;
+    R.x = bt->x; R.lam = bt->lambda; R.mask = bt->mask; R.gen_mask = bt->gen_mask;
+    R.pd_scale = bt->pd_scale; R.obj_weight = bt->obj_weight; R.sigma = bt->obj_factor;
+    R.f = f; R.grad = grad; R.gh = gh; R.jval = jval; R.hval = hval;
+    R.tab = tab;
+    return R;
+}
+
 // One evaluation call.  With the internal workspace, the call is ordered after the last use of
 // that workspace on any other stream (ws_acquire_locked).
 exago_status eval(exago_net *net, const exago_batch *bt, double *f, double *grad, double *gh,
@@ -669,6 +726,14 @@ exago_status eval(exago_net *net, const exago_batch *bt, double *f, double *grad
     exago_status s = check_batch(net, bt, hval != nullptr);
     if (s != EXAGO_OK || bt->B == 0) return s;
     std::lock_guard<std::mutex> lk(net->mu);
+    const StateBlock sb = hook ? StateBlock{} : state_block(net, bt->B);
+    if (sb.nt) {   // one kernel, no scratch
+        EvalReq R = request(bt, f, grad, gh, jval, hval, tab);
+        R.stage_cap = sb.cap;
+        const int e = launch_eval_state(net->dev, R, sb.nt, sb.smem, bt->stream);
+        if (e != 0) return cuda_fail((cudaError_t)e, "block-per-state launch");
+        return EXAGO_OK;
+    }
     const Resolved rs = resolve(net, bt->B);
     void *ws = bt->workspace;
     const bool needs_ws = gh || jval || hval || rs.schedule == EXAGO_SCHED_PERSISTENT;
@@ -687,14 +752,9 @@ exago_status eval_locked(exago_net *net, const exago_batch *bt, double *f, doubl
                          double *gh, double *jval, double *hval, ProfileHook *hook,
                          bool allow_graph, const StateTab *tab, const Resolved &rs, void *ws) {
     exago_status s = EXAGO_OK;
-    EvalReq R{};
-    R.B = bt->B;
-    R.x = bt->x; R.lam = bt->lambda; R.mask = bt->mask; R.gen_mask = bt->gen_mask;
-    R.pd_scale = bt->pd_scale; R.obj_weight = bt->obj_weight; R.sigma = bt->obj_factor;
-    R.f = f; R.grad = grad; R.gh = gh; R.jval = jval; R.hval = hval;
+    EvalReq R = request(bt, f, grad, gh, jval, hval, tab);
     R.stage_recs = rs.stage_recs;
     R.stage_cap = rs.stage_cap;
-    R.tab = tab;
     cudaStream_t stream = (cudaStream_t)bt->stream;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t ce = cudaStreamIsCapturing(stream, &cap);

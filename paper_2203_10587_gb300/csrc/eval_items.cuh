@@ -723,7 +723,8 @@ __device__ __forceinline__ bool bulk_wait(unsigned long long *mbar, unsigned par
 // When the row segments fit (after the components, if used), every row entry is written to
 // shared memory and the group copies the four segments out with coalesced stores; otherwise
 // the rows go straight to global memory.  Contains G::sync(): call from every thread.
-template <int WANT, class G>
+// SREC: scr itself is in shared memory (the block-per-state schedule).
+template <int WANT, class G, bool SREC = false>
 __device__ __forceinline__ void bus_tile(const DevNet &N, const EvalReq &R, int b, int i0,
                                          const double *scr, double *stage, int cap,
                                          const BulkCtx *bk = nullptr, unsigned *phase = nullptr) {
@@ -772,7 +773,7 @@ __device__ __forceinline__ void bus_tile(const DevNet &N, const EvalReq &R, int 
         *phase ^= 1u;
         if (i < i1 && ok) bus_item<WANT, true>(N, R, b, i, stage, S0, T.template of<WANT>(N, i));
     } else if (i < i1) {
-        bus_item<WANT, false>(N, R, b, i, scr, 0, T.template of<WANT>(N, i));
+        bus_item<WANT, SREC>(N, R, b, i, scr, 0, T.template of<WANT>(N, i));
     }
     if (staged) {
         G::sync();
@@ -887,12 +888,13 @@ __device__ __forceinline__ void obj_lanes(const DevNet &N, const EvalReq &R, int
 // calling warp): levels 128, 64 and 32 in registers (lane l holds lanes l + 32 j), then 16 .. 1
 // by shuffles, each level adding part[v + w] to part[v] for v < w as obj_block does, so the
 // result is bitwise obj_block's.  Writes f[b].  partials were written by other CTAs of the launch
-// (read through L2).
+// (read through L2; SMEM: by this block, in shared memory).
+template <bool SMEM = false>
 __device__ __forceinline__ void obj_tree_warp(const EvalReq &R, int b, const double *partials) {
     const int l = threadIdx.x & 31;
     double p[8];
 #pragma unroll
-    for (int j = 0; j < 8; j++) p[j] = __ldcg(partials + l + 32 * j);
+    for (int j = 0; j < 8; j++) p[j] = SMEM ? partials[l + 32 * j] : __ldcg(partials + l + 32 * j);
 #pragma unroll
     for (int j = 0; j < 4; j++) p[j] += p[j + 4];
     p[0] += p[2];

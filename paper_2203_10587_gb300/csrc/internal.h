@@ -230,6 +230,12 @@ int persist_w_allow_stage();
 // Shared memory of a bus tile (eval_items.cuh, bus_tile): its records and its row segments.  The
 // largest tile's need in doubles, capped at kStageMaxDoubles; a tile above the cap reads its
 // records from global memory and writes its rows directly.
+// Block-per-state schedule (state_block.cu): a state's records and staged rows in one block's
+// shared memory.  nt: 64 or 256 threads; smem: bytes, at most kStateMaxBytes.
+constexpr int kStateMaxBytes = 200 << 10;
+int state_allow_smem();
+int launch_eval_state(const DevNet &net, const EvalReq &req, int nt, size_t smem, void *stream);
+
 constexpr int kStageMaxDoubles = 9216;   // 72 KB
 // The persistent schedule's ring slot of one state: NCOMP x nslot doubles of branch-end records,
 // then the kObjLanes partial sums of the state's objective (256 virtual lanes).
