@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include "int_mul.cuh"
 #include "internal.h"
 
 namespace exago {
@@ -160,20 +161,23 @@ struct End {
 };
 
 // Gss2 = 2 Gss and Bss2 = 2 Bss (network tables); Vu2 = Vu^2 and VV = Vu Vv from the caller.
-template <bool DERIV>
+// mul: how products are formed (int_mul.cuh); the caller has noted Vu, Vv and VV as needed.
+template <bool DERIV, typename M>
 __device__ __forceinline__ End end_terms(double Gss, double Bss, double Gss2, double Bss2,
                                          double A, double C, double Vu, double Vv, double Vu2,
-                                         double VV) {
+                                         double VV, M &mul) {
     End e;
-    e.qa = VV * A;                 //  Vu Vv A
-    e.pa = -(VV * C);              // -Vu Vv C
+    mul.need(A);
+    mul.need(C);
+    e.qa = mul(VV, A);             //  Vu Vv A
+    e.pa = -mul(VV, C);            // -Vu Vv C
     e.P = fma(Gss, Vu2, e.qa);
     e.Q = fma(-Bss, Vu2, -e.pa);
     if (DERIV) {
-        e.pv = Vu * A;
-        e.qv = Vu * C;
-        e.pu = fma(Gss2, Vu, Vv * A);
-        e.qu = fma(-Bss2, Vu, Vv * C);
+        e.pv = mul(Vu, A);
+        e.qv = mul(Vu, C);
+        e.pu = fma(Gss2, Vu, mul(Vv, A));
+        e.qu = fma(-Bss2, Vu, mul(Vv, C));
     }
     return e;
 }
@@ -191,21 +195,24 @@ struct EndHess {
     double W1, W2, tK, hau, huu, huv;   // tK = 2 mu K
 };
 
+template <typename M>
 __device__ __forceinline__ EndHess end_hess(const End &e, double Gss2, double Bss2, double A,
                                             double C, double K, double Vu, double Vv,
-                                            double lamP, double lamQ, double mu) {
+                                            double lamP, double lamQ, double mu, M &mul) {
     EndHess h;
+    mul.need(e.pu);
+    mul.need(e.qu);
     const double mu2 = twice(mu);
     const double wP = fma(mu2, e.P, lamP);
     const double wQ = fma(mu2, e.Q, lamQ);
     h.W1 = fma(wP, A, wQ * C);
     h.W2 = fma(wQ, A, -(wP * C));
-    const double E = fma(A, e.qu, -(C * e.pu));
-    const double F = fma(e.pu, A, e.qu * C);
+    const double E = fma(A, e.qu, -mul(C, e.pu));
+    const double F = fma(e.pu, A, mul(e.qu, C));
     h.tK = mu2 * K;
     const double mu2Vu = mu2 * Vu;
     h.hau = Vv * fma(mu2Vu, E, h.W2);             // 2 mu Vu Vv E + Vv W2
-    const double S = fma(e.pu, e.pu, e.qu * e.qu);
+    const double S = fma(e.pu, e.pu, mul(e.qu, e.qu));
     h.huu = fma(mu2, S, fma(wP, Gss2, -(wQ * Bss2)));
     h.huv = fma(mu2Vu, F, h.W1);
     return h;
@@ -331,8 +338,9 @@ __device__ __forceinline__ void branch_item(const DevNet &N, const EvalReq &R, i
     const double *lb = WH ? st_lam(N, R, b) : nullptr;
     const double K = WH ? __ldg(N.Kft + l) : 0.0;    // A^2 + C^2 = G^2 + B^2 at both ends
     EndHess hf{}, ht{};
+    Mul<false> mul;
     {
-        const End ef = end_terms<DERIV>(Gff, Bff, Gff2, Bff2, Af, Cf, Vf, Vt, Vf2, VV);
+        const End ef = end_terms<DERIV>(Gff, Bff, Gff2, Bff2, Af, Cf, Vf, Vt, Vf2, VV, mul);
         if (WG && ghb) *hrf = fma(ef.P, ef.P, ef.Q * ef.Q);
         if (WG || WJ) {
             put2<PS>(rf, SC_PA, ef.pa, ef.pu); put2<PS>(rf, SC_PV, ef.pv, ef.qa); put2<PS>(rf, SC_QU, ef.qu, ef.qv);
@@ -340,10 +348,10 @@ __device__ __forceinline__ void branch_item(const DevNet &N, const EvalReq &R, i
         if (WJ) store_hrow(Jf, ef, fb < tb);
         if (WH)
             hf = end_hess(ef, Gff2, Bff2, Af, Cf, K, Vf, Vt, __ldg(lb + fb), __ldg(lb + nb + fb),
-                          __ldg(lb + 2 * nb + l));
+                          __ldg(lb + 2 * nb + l), mul);
     }
     {
-        const End et = end_terms<DERIV>(Gtt, Btt, Gtt2, Btt2, At, Ct, Vt, Vf, Vt2, VV);
+        const End et = end_terms<DERIV>(Gtt, Btt, Gtt2, Btt2, At, Ct, Vt, Vf, Vt2, VV, mul);
         if (WG && ghb) *hrt = fma(et.P, et.P, et.Q * et.Q);
         if (WG || WJ) {
             put2<PS>(rt, SC_PA, et.pa, et.pu); put2<PS>(rt, SC_PV, et.pv, et.qa); put2<PS>(rt, SC_QU, et.qu, et.qv);
@@ -351,7 +359,7 @@ __device__ __forceinline__ void branch_item(const DevNet &N, const EvalReq &R, i
         if (WJ) store_hrow(Jt, et, tb < fb);
         if (WH)
             ht = end_hess(et, Gtt2, Btt2, At, Ct, K, Vt, Vf, __ldg(lb + tb), __ldg(lb + nb + tb),
-                          __ldg(lb + 2 * nb + nl + l));
+                          __ldg(lb + 2 * nb + nl + l), mul);
     }
     if (WH) {
         const BranchHess h = branch_hess(hf, ht, Vf, Vt, Vf2, Vt2, VV);
