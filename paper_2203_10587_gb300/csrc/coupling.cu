@@ -10,8 +10,8 @@
 // gather over each state's children, in a fixed order (no atomics):
 //     (C^T nu)[b][Pg_k] = [p(b) >= 0] nu[b][k] - sum over children c of b of nu[c][k].
 // States with few children are summed by one thread per (state, generator); a state with many
-// children (the base case of a contingency or scenario batch) is summed by blocks of 8 generators
-// whose 32 rows of threads take every 32nd child of the list staged in shared memory and then
+// children (the base case of a contingency or scenario batch) is summed by blocks of 4 generators
+// whose 64 rows of threads take every 64th child of the list staged in shared memory and then
 // reduce in a fixed tree.
 #include <cuda_runtime.h>
 
@@ -36,8 +36,9 @@ namespace {
 
 using exago::set_last_error;
 
-// A state with more children than this is reduced by blocks of (8 generators x 32 child lanes).
+// A state with more children than this is reduced by blocks of kHeavyCols x kHeavyRows.
 constexpr int kHeavyChildren = 8;
+constexpr int kHeavyCols = 4, kHeavyRows = 64;   // generators x child lanes of such a block
 constexpr int kMaxGridY = 65535;
 // Children of a heavy state staged in shared memory per pass.
 constexpr int kStageChildren = 2048;
@@ -75,18 +76,61 @@ __device__ __forceinline__ void put(double *o, double v, int accumulate) {
     *o = accumulate ? *o + v : v;
 }
 
-// Block (256 threads) per (listed state, kRowSpan generators): its own row's multiplier minus its
-// children's, the children in ascending order.  The state's child range is uniform over the block.
-__global__ void __launch_bounds__(256) k_coupling_jtv_light(
-    const int *__restrict__ light, int j0, const int *__restrict__ parent,
-    const int *__restrict__ cptr, const int *__restrict__ cidx, int ng,
-    const double *__restrict__ nu, double *out, int64_t ldo, int accumulate) {
-    const int s = __ldg(light + j0 + blockIdx.y);
-    const bool own = __ldg(parent + s) >= 0;
-    const int c0 = __ldg(cptr + s), c1 = __ldg(cptr + s + 1);
-    const double *ns = nu + (int64_t)s * ng;
-    double *os = out + (int64_t)s * ldo;
-    const int k0 = blockIdx.x * kRowSpan + threadIdx.x;
+struct JtvArgs {
+    const int *light, *heavy, *parent, *cptr, *cidx;
+    int nheavy, hblocks, lblocks, ng, accumulate;   // hblocks, lblocks: blocks of one state
+    const double *nu;
+    double *out;
+    int64_t ldo;
+};
+
+// One launch for all states (256 threads a block): first the heavy ones, hblocks blocks of
+// kHeavyCols generators each, then the light ones, lblocks blocks of kRowSpan generators each.
+//   * heavy: the state's children are staged in shared memory, thread row ty sums children ty,
+//     ty + kHeavyRows, ... (independent loads), and the partial sums are reduced by a fixed halving
+//     tree.  A 512-state star: 8 children a thread in one batch of loads; with 8 generators x 32
+//     rows they were two, in a launch of its own (15.6 us the two launches);
+//   * light: the state's own row minus its children's, in ascending order.
+__global__ void __launch_bounds__(256) k_coupling_jtv(const JtvArgs A) {
+    __shared__ int kids[kStageChildren];
+    __shared__ double part[kHeavyRows][kHeavyCols + 1];
+    const int tid = threadIdx.x, ng = A.ng;
+    const int64_t heavy_blocks = (int64_t)A.nheavy * A.hblocks;
+    if ((int64_t)blockIdx.x < heavy_blocks) {
+        const int tx = tid % kHeavyCols, ty = tid / kHeavyCols;
+        const int s = __ldg(A.heavy + blockIdx.x / A.hblocks);
+        const int k = (blockIdx.x % A.hblocks) * kHeavyCols + tx;
+        const int c0 = __ldg(A.cptr + s), c1 = __ldg(A.cptr + s + 1);
+        double acc = 0.0;
+        for (int base = c0; base < c1; base += kStageChildren) {
+            const int cnt = min(kStageChildren, c1 - base);
+            __syncthreads();   // the previous pass is done with kids
+            for (int j = tid; j < cnt; j += 256) kids[j] = __ldg(A.cidx + base + j);
+            __syncthreads();
+            if (k < ng) {
+#pragma unroll 8
+                for (int j = ty; j < cnt; j += kHeavyRows) acc += __ldg(A.nu + (int64_t)kids[j] * ng + k);
+            }
+        }
+        part[ty][tx] = acc;
+        __syncthreads();
+        for (int h = kHeavyRows / 2; h >= 1; h >>= 1) {
+            if (ty < h) part[ty][tx] += part[ty + h][tx];
+            __syncthreads();
+        }
+        if (ty == 0 && k < ng) {
+            const double own = __ldg(A.parent + s) >= 0 ? __ldg(A.nu + (int64_t)s * ng + k) : 0.0;
+            put(A.out + (int64_t)s * A.ldo + k, own - part[0][tx], A.accumulate);
+        }
+        return;
+    }
+    const int64_t blk = (int64_t)blockIdx.x - heavy_blocks;
+    const int s = __ldg(A.light + blk / A.lblocks);
+    const bool own = __ldg(A.parent + s) >= 0;
+    const int c0 = __ldg(A.cptr + s), c1 = __ldg(A.cptr + s + 1);
+    const double *ns = A.nu + (int64_t)s * ng;
+    double *os = A.out + (int64_t)s * A.ldo;
+    const int k0 = (int)(blk % A.lblocks) * kRowSpan + tid;
     double v[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; u++) {
@@ -94,7 +138,7 @@ __global__ void __launch_bounds__(256) k_coupling_jtv_light(
         v[u] = own && k < ng ? __ldg(ns + k) : 0.0;
     }
     for (int c = c0; c < c1; c++) {
-        const double *nc = nu + (int64_t)__ldg(cidx + c) * ng;
+        const double *nc = A.nu + (int64_t)__ldg(A.cidx + c) * ng;
 #pragma unroll
         for (int u = 0; u < kUnroll; u++) {
             const int k = k0 + u * 256;
@@ -104,46 +148,11 @@ __global__ void __launch_bounds__(256) k_coupling_jtv_light(
 #pragma unroll
     for (int u = 0; u < kUnroll; u++) {
         const int k = k0 + u * 256;
-        if (k < ng) put(os + k, v[u], accumulate);
+        if (k < ng) put(os + k, v[u], A.accumulate);
     }
 }
 
-// Block (8 x 32) per (listed state, 8 generators): the state's children are staged in shared
-// memory, thread row ty sums children ty, ty + 32, ... (independent loads), and the 32 partial
-// sums are reduced by a fixed halving tree.
-__global__ void __launch_bounds__(256) k_coupling_jtv_heavy(
-    const int *__restrict__ heavy, int h0, const int *__restrict__ parent,
-    const int *__restrict__ cptr, const int *__restrict__ cidx, int ng,
-    const double *__restrict__ nu, double *out, int64_t ldo, int accumulate) {
-    __shared__ int kids[kStageChildren];
-    __shared__ double part[32][9];
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 8 + tx;
-    const int s = __ldg(heavy + h0 + blockIdx.y);
-    const int k = blockIdx.x * 8 + tx;
-    const int c0 = __ldg(cptr + s), c1 = __ldg(cptr + s + 1);
-    double acc = 0.0;
-    for (int base = c0; base < c1; base += kStageChildren) {
-        const int cnt = min(kStageChildren, c1 - base);
-        __syncthreads();   // the previous pass is done with kids
-        for (int j = tid; j < cnt; j += 256) kids[j] = __ldg(cidx + base + j);
-        __syncthreads();
-        if (k < ng) {
-#pragma unroll 8
-            for (int j = ty; j < cnt; j += 32) acc += __ldg(nu + (int64_t)kids[j] * ng + k);
-        }
-    }
-    part[ty][tx] = acc;
-    __syncthreads();
-    for (int h = 16; h >= 1; h >>= 1) {
-        if (ty < h) part[ty][tx] += part[ty + h][tx];
-        __syncthreads();
-    }
-    if (ty == 0 && k < ng) {
-        const double own = __ldg(parent + s) >= 0 ? __ldg(nu + (int64_t)s * ng + k) : 0.0;
-        put(out + (int64_t)s * ldo + k, own - part[0][tx], accumulate);
-    }
-}
-
+// Blocks along a row of ng values: one 256-thread block per kRowSpan values.
 exago_status check_call(exago_coupling_t c) {
     if (!c) return set_last_error(EXAGO_EINVAL, "coupling is NULL");
     if (!c->on_device)
@@ -320,17 +329,16 @@ exago_status exago_eval_coupling_jtv(exago_coupling_t c, const double *nu, doubl
     if (ldo < c->ng) return set_last_error(EXAGO_EINVAL, "ldo < ng");
     cudaStream_t s = (cudaStream_t)stream;
     const int nlight = (int)c->light.size(), nheavy = (int)c->heavy.size();
-    for (int j0 = 0; j0 < nlight; j0 += kMaxGridY) {
-        const int nj = std::min(kMaxGridY, nlight - j0);
-        k_coupling_jtv_light<<<dim3(row_blocks(c->ng), nj), 256, 0, s>>>(
-            c->d_light, j0, c->d_parent, c->d_child_ptr, c->d_child_idx, c->ng, nu, out, ldo,
-            accumulate ? 1 : 0);
-    }
-    for (int h0 = 0; h0 < nheavy; h0 += kMaxGridY) {
-        const int nh = std::min(kMaxGridY, nheavy - h0);
-        k_coupling_jtv_heavy<<<dim3((c->ng + 7) / 8, nh), dim3(8, 32), 0, s>>>(
-            c->d_heavy, h0, c->d_parent, c->d_child_ptr, c->d_child_idx, c->ng, nu, out, ldo,
-            accumulate ? 1 : 0);
+    // states of one launch, so that its blocks fit the grid (2^31 - 1)
+    const int hb = (c->ng + kHeavyCols - 1) / kHeavyCols, lb = (int)row_blocks(c->ng);
+    const int hmax = std::max(1, (1 << 30) / hb), lmax = std::max(1, (1 << 30) / lb);
+    for (int h0 = 0, l0 = 0; h0 < nheavy || l0 < nlight;) {
+        const int nh = std::min(hmax, nheavy - h0), nl = std::min(lmax, nlight - l0);
+        const JtvArgs A{c->d_light + l0, c->d_heavy + h0, c->d_parent, c->d_child_ptr, c->d_child_idx,
+                        nh, hb, lb, c->ng, accumulate ? 1 : 0, nu, out, ldo};
+        k_coupling_jtv<<<(unsigned)(nh * hb + nl * lb), 256, 0, s>>>(A);
+        h0 += nh;
+        l0 += nl;
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)

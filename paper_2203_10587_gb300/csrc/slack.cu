@@ -2,13 +2,14 @@
 // Sec. III, Fig. 2).  Each slack z_k >= 0 sits at one bus, in the P or the Q balance, with sign
 // +1 or -1 and a linear cost: it adds sign z_k to that balance and w cost_k z_k to the objective;
 // its Jacobian column is the constant sign in that row and the Hessian gets nothing.  The terms
-// are applied to a finished evaluation (exago_eval_* outputs) by three small kernels:
-//   * rows: one thread per (balance row with slacks, group of 8 states) adds the row's slacks in
-//     ascending slack order to each state's value (the same additions, in the same order, as the
-//     definition);
-//   * objective: one block per state sums cost_k z_k (four partial sums per thread, then a fixed
-//     256-lane tree) and adds w times the sum to f; the gradient w cost_k by its own kernel;
-//   * transpose: one thread per (state, slack) gathers sign_k v[row_k].
+// are applied to a finished evaluation (exago_eval_* outputs) by one launch, whose blocks do one of
+// three things for one state:
+//   * objective: one block sums cost_k z_k (four partial sums per thread, then a fixed 256-lane
+//     tree) and adds w times the sum to f;
+//   * rows: a thread per balance row with slacks adds the row's slacks in ascending slack order (the
+//     same additions, in the same order, as the definition);
+//   * gradient w cost_k.
+// The transpose is a second kernel: sign_k v[row_k], four slacks per thread.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -17,6 +18,7 @@
 #include <string>
 #include <vector>
 
+#include "int_mul.cuh"
 #include "internal.h"
 
 struct exago_slack {
@@ -27,100 +29,135 @@ struct exago_slack {
     std::vector<double> cost;
     std::vector<int> grow;              // [nz] balance row of each slack: row nb + bus
     std::vector<int> rptr, rlist, used; // CSR of the slacks by balance row; rows that have some
-    int *d_int = nullptr;               // grow, sign, rptr, rlist, used
+    int *d_int = nullptr;               // rows with slacks and the end (int2); grow and rlist as index << 1 |
+                                        // negative
     double *d_cost = nullptr;
     void *d_mem = nullptr;
 };
 
 namespace {
 
+using exago::int_mul;
+using exago::mul_window;
 using exago::set_last_error;
 
 constexpr int kLanes = 256;
 constexpr int kMaxGridY = 65535;
+constexpr int kPart = 1024;   // gradient entries of one block
 
-// Balance rows: one thread per (balance row with slacks, group of kGroup states).  The row's slack
-// list is read once for the group; each state's value gets the row's slacks in ascending order
-// (the definition's additions in the definition's order), the group's loads issued together.
-constexpr int kGroup = 8;
-__global__ void __launch_bounds__(128) k_slack_rows(const int *__restrict__ used, int nused,
-                                                    const int *__restrict__ rptr,
-                                                    const int *__restrict__ rlist,
-                                                    const int *__restrict__ sign, int nz, int b0,
-                                                    int nB, const double *__restrict__ z,
-                                                    double *gh, int64_t ldgh) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= nused) return;
-    const int g0 = b0 + blockIdx.y * kGroup;
-    const int ns = min(kGroup, b0 + nB - g0);
-    const int r = __ldg(used + j);
-    double v[kGroup];
-#pragma unroll
-    for (int t = 0; t < kGroup; t++)
-        if (t < ns) v[t] = gh[(int64_t)(g0 + t) * ldgh + r];
-    for (int q = __ldg(rptr + r), q1 = __ldg(rptr + r + 1); q < q1; q++) {
-        const int k = __ldg(rlist + q);
-        const double sk = __ldg(sign + k);
-#pragma unroll
-        for (int t = 0; t < kGroup; t++)
-            if (t < ns) v[t] += sk * __ldg(z + (int64_t)(g0 + t) * nz + k);
-    }
-#pragma unroll
-    for (int t = 0; t < kGroup; t++)
-        if (t < ns) gh[(int64_t)(g0 + t) * ldgh + r] = v[t];
+// A table entry is an index << 1 | (sign is -1).  The sign is applied to the bits: a multiplication
+// by -1 takes the FP64 pipe 64 cycles a warp, which bounded the first version of both kernels.
+__device__ __forceinline__ double signed_by(double v, unsigned code) {
+    return __hiloint2double(__double2hiint(v) ^ (int)(code << 31), __double2loint(v));
 }
 
-// Objective: one block per state; each thread keeps four partial sums over slacks t, t + 256,
-// t + 512, t + 768, then t + 1024, ... (independent loads in flight), combined in a fixed order
-// and then over a fixed 256-lane tree.
-__global__ void __launch_bounds__(kLanes) k_slack_obj(const double *__restrict__ cost, int nz,
-                                                      int b0, const double *__restrict__ z,
-                                                      const double *__restrict__ obj_weight,
-                                                      double *f) {
+// Out of line, so that no FP64 multiplication is issued for every product beside the integer one.
+__device__ __noinline__ double fp_mul(double x, double y) { return x * y; }
+
+constexpr int kStates = 4;    // states of one block of rows or gradient: they share its tables
+
+struct SlackArgs {
+    const int2 *rows;               // balance rows with slacks: row, first entry (and the end)
+    const unsigned *rcode;          // slack << 1 | negative, by row
+    int nused, nz, b0, nB, row_blocks, grad_blocks;
+    const double *cost, *z, *obj_weight;
+    double *gh, *f, *grad_z;
+    int64_t ldgh;
+};
+
+// For the states b0 + kStates y ..: blocks x < kStates do the objective of one state each, then
+// row_blocks blocks the rows and grad_blocks the gradient of all of them.  One launch in place of
+// three, each of which waited for the one before.  Bound by the FP64 pipe (an addition a slack
+// for the rows and a multiply-add for the objective: 18 us on 2,000 buses x 512 states, 10,766
+// slacks a state), so the gradient's products go to the integer pipe.  69 us in three launches
+// with FP64 sign and gradient products, 41 now.
+__global__ void __launch_bounds__(kLanes) k_slack_apply(const SlackArgs A) {
     __shared__ double part[kLanes];
-    const int b = b0 + blockIdx.x;
-    const double *zb = z + (int64_t)b * nz;
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    int k = threadIdx.x;
-    for (; k + 3 * kLanes < nz; k += 4 * kLanes) {
-        a0 = fma(__ldg(cost + k), __ldg(zb + k), a0);
-        a1 = fma(__ldg(cost + k + kLanes), __ldg(zb + k + kLanes), a1);
-        a2 = fma(__ldg(cost + k + 2 * kLanes), __ldg(zb + k + 2 * kLanes), a2);
-        a3 = fma(__ldg(cost + k + 3 * kLanes), __ldg(zb + k + 3 * kLanes), a3);
-    }
-    for (; k < nz; k += kLanes) a0 = fma(__ldg(cost + k), __ldg(zb + k), a0);
-    part[threadIdx.x] = (a0 + a1) + (a2 + a3);
-    __syncthreads();
-    for (int h = kLanes / 2; h > 0; h >>= 1) {
-        if (threadIdx.x < h) part[threadIdx.x] += part[threadIdx.x + h];
+    const int tid = threadIdx.x, bs = A.b0 + kStates * blockIdx.y, nz = A.nz;
+    const int ns = min(kStates, A.b0 + A.nB - bs);
+    int x = blockIdx.x;
+    if (x < kStates) {
+        if (!A.f || x >= ns) return;
+        const int b = bs + x;
+        const double *zb = A.z + (int64_t)b * nz;
+        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+        int k = tid;
+        for (; k + 3 * kLanes < nz; k += 4 * kLanes) {
+            a0 = fma(__ldg(A.cost + k), __ldg(zb + k), a0);
+            a1 = fma(__ldg(A.cost + k + kLanes), __ldg(zb + k + kLanes), a1);
+            a2 = fma(__ldg(A.cost + k + 2 * kLanes), __ldg(zb + k + 2 * kLanes), a2);
+            a3 = fma(__ldg(A.cost + k + 3 * kLanes), __ldg(zb + k + 3 * kLanes), a3);
+        }
+        for (; k < nz; k += kLanes) a0 = fma(__ldg(A.cost + k), __ldg(zb + k), a0);
+        part[tid] = (a0 + a1) + (a2 + a3);
         __syncthreads();
+        for (int h = kLanes / 2; h > 0; h >>= 1) {
+            if (tid < h) part[tid] += part[tid + h];
+            __syncthreads();
+        }
+        if (tid == 0) A.f[b] = fma(A.obj_weight ? __ldg(A.obj_weight + b) : 1.0, part[0], A.f[b]);
+        return;
     }
-    if (threadIdx.x == 0) f[b] = fma(obj_weight ? __ldg(obj_weight + b) : 1.0, part[0], f[b]);
-}
-
-// Gradient w cost_k: blocks of 256 threads along each state's slacks, four values per thread.
-__global__ void __launch_bounds__(256) k_slack_grad(const double *__restrict__ cost, int nz,
-                                                    int b0, const double *__restrict__ obj_weight,
-                                                    double *__restrict__ grad_z) {
-    const int b = b0 + blockIdx.y;
-    const double w = obj_weight ? __ldg(obj_weight + b) : 1.0;
-    double *gb = grad_z + (int64_t)b * nz;
-    const int k0 = blockIdx.x * 1024 + threadIdx.x;
+    x -= kStates;
+    if (x < A.row_blocks) {
+        const int j = x * kLanes + tid;
+        if (j >= A.nused) return;
+        const int2 row = __ldg(A.rows + j);
+        const int q1 = __ldg(&A.rows[j + 1].y);
+        double *g = A.gh + (int64_t)bs * A.ldgh + row.x;
+        const double *zb = A.z + (int64_t)bs * nz;
+        double v[kStates];
 #pragma unroll
-    for (int u = 0; u < 4; u++) {
-        const int k = k0 + u * 256;
-        if (k < nz) gb[k] = w * __ldg(cost + k);
+        for (int t = 0; t < kStates; t++) v[t] = t < ns ? g[t * A.ldgh] : 0.0;
+        for (int q = row.y; q < q1; q += 2) {        // two entries' loads in flight
+            const unsigned c0 = __ldg(A.rcode + q), c1 = q + 1 < q1 ? __ldg(A.rcode + q + 1) : 0;
+            double t0[kStates], t1[kStates];
+#pragma unroll
+            for (int t = 0; t < kStates; t++) {
+                t0[t] = t < ns ? __ldg(zb + (int64_t)t * nz + (c0 >> 1)) : 0.0;
+                t1[t] = t < ns && q + 1 < q1 ? __ldg(zb + (int64_t)t * nz + (c1 >> 1)) : 0.0;
+            }
+#pragma unroll
+            for (int t = 0; t < kStates; t++) v[t] += signed_by(t0[t], c0);
+            if (q + 1 < q1)
+#pragma unroll
+                for (int t = 0; t < kStates; t++) v[t] += signed_by(t1[t], c1);
+        }
+#pragma unroll
+        for (int t = 0; t < kStates; t++)
+            if (t < ns) g[t * A.ldgh] = v[t];
+        return;
+    }
+    x -= A.row_blocks;
+#pragma unroll
+    for (int u = 0; u < kPart / kLanes; u++) {
+        const int k = x * kPart + u * kLanes + tid;
+        if (k >= nz) break;
+        const double c = __ldg(A.cost + k);
+        for (int t = 0; t < ns; t++) {
+            const double w = A.obj_weight ? __ldg(A.obj_weight + bs + t) : 1.0;
+            A.grad_z[(int64_t)(bs + t) * nz + k] = mul_window(w) && mul_window(c) ? int_mul(w, c)
+                                                                                  : fp_mul(w, c);
+        }
     }
 }
 
-__global__ void __launch_bounds__(256) k_slack_jtv(const int *__restrict__ grow,
-                                                   const int *__restrict__ sign, int nz, int b0,
+// out[b][k] = sign_k v[b][row_k]: every load of a thread's four slacks before its first store.
+__global__ void __launch_bounds__(256) k_slack_jtv(const unsigned *__restrict__ gcode, int nz, int b0,
                                                    const double *__restrict__ v, int64_t ldv,
-                                                   double *out) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nz) return;
-    const int b = b0 + blockIdx.y;
-    out[(int64_t)b * nz + k] = __ldg(sign + k) * __ldg(v + (int64_t)b * ldv + __ldg(grow + k));
+                                                   double *__restrict__ out) {
+    const int b = b0 + blockIdx.y, k0 = blockIdx.x * 1024 + threadIdx.x;
+    const double *vb = v + (int64_t)b * ldv;
+    double *ob = out + (int64_t)b * nz;
+    unsigned c[4];
+    double t[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) c[u] = k0 + u * 256 < nz ? __ldg(gcode + k0 + u * 256) : 0;
+#pragma unroll
+    for (int u = 0; u < 4; u++) t[u] = k0 + u * 256 < nz ? __ldg(vb + (c[u] >> 1)) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 4; u++)
+        if (k0 + u * 256 < nz) ob[k0 + u * 256] = signed_by(t[u], c[u]);
 }
 
 exago_status check_call(exago_slack_t s, const exago_batch *bt) {
@@ -197,11 +234,12 @@ exago_status exago_slack_create(exago_net_t net, int nz, const int *bus, const i
                                                    : "make the net's device current before the call");
         }
         std::vector<int> ints;
-        ints.insert(ints.end(), s->grow.begin(), s->grow.end());
-        ints.insert(ints.end(), s->sign.begin(), s->sign.end());
-        ints.insert(ints.end(), s->rptr.begin(), s->rptr.end());
-        ints.insert(ints.end(), s->rlist.begin(), s->rlist.end());
-        ints.insert(ints.end(), s->used.begin(), s->used.end());
+        for (int r : s->used)
+            for (int v : {r, s->rptr[r]}) ints.push_back(v);
+        for (int v : {0, nz}) ints.push_back(v);   // the rows' end
+        auto code = [&](int index, int k) { return (int)((unsigned)index << 1 | (unsigned)(s->sign[k] < 0)); };
+        for (int k = 0; k < nz; k++) ints.push_back(code(s->grow[k], k));
+        for (int k : s->rlist) ints.push_back(code(k, k));
         const size_t ibytes = (ints.size() * sizeof(int) + 255) / 256 * 256;
         const size_t bytes = ibytes + std::max<size_t>((size_t)nz, 1) * sizeof(double);
         e = exago::dev_malloc(&s->d_mem, bytes);
@@ -250,17 +288,15 @@ exago_status exago_eval_slack(exago_slack_t s, const exago_batch *bt, const doub
     if (gh && ldgh < 2 * s->nb) return set_last_error(EXAGO_EINVAL, "ldgh < 2 nb");
     cudaStream_t stream = (cudaStream_t)bt->stream;
     const int nused = (int)s->used.size();
-    const int *grow = s->d_int, *sign = grow + s->nz, *rptr = sign + s->nz;
-    const int *rlist = rptr + 2 * s->nb + 1, *used = rlist + s->nz;
-    for (int b0 = 0; b0 < bt->B; b0 += kMaxGridY) {
-        const int nB = std::min(kMaxGridY, bt->B - b0);
-        if (gh && nused > 0)
-            k_slack_rows<<<dim3((nused + 127) / 128, (nB + kGroup - 1) / kGroup), 128, 0, stream>>>(
-                used, nused, rptr, rlist, sign, s->nz, b0, nB, z, gh, ldgh);
-        if (f) k_slack_obj<<<nB, kLanes, 0, stream>>>(s->d_cost, s->nz, b0, z, bt->obj_weight, f);
-        if (grad_z)
-            k_slack_grad<<<dim3((s->nz + 1023) / 1024, nB), 256, 0, stream>>>(
-                s->d_cost, s->nz, b0, bt->obj_weight, grad_z);
+    SlackArgs A{(const int2 *)s->d_int, (const unsigned *)s->d_int + 2 * (nused + 1) + s->nz, nused,
+                s->nz, 0, 0, gh ? (nused + kLanes - 1) / kLanes : 0,
+                grad_z ? (s->nz + kPart - 1) / kPart : 0,
+                s->d_cost, z, bt->obj_weight, gh, f, grad_z, ldgh};
+    for (int b0 = 0; b0 < bt->B && (gh || f || grad_z); b0 += kMaxGridY) {
+        A.b0 = b0;
+        A.nB = std::min(kMaxGridY, bt->B - b0);
+        k_slack_apply<<<dim3(kStates + A.row_blocks + A.grad_blocks, (A.nB + kStates - 1) / kStates),
+                        kLanes, 0, stream>>>(A);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
@@ -287,11 +323,10 @@ exago_status exago_eval_slack_jtv(exago_slack_t s, const exago_batch *bt, const 
     if (st != EXAGO_OK || bt->B == 0 || s->nz == 0) return st;
     if (!v || !out) return set_last_error(EXAGO_EINVAL, "v or out is NULL");
     if (ldv < 2 * s->nb) return set_last_error(EXAGO_EINVAL, "ldv < 2 nb");
-    const int *grow = s->d_int, *sign = grow + s->nz;
     for (int b0 = 0; b0 < bt->B; b0 += kMaxGridY) {
         const int nB = std::min(kMaxGridY, bt->B - b0);
-        k_slack_jtv<<<dim3((s->nz + 255) / 256, nB), 256, 0, (cudaStream_t)bt->stream>>>(
-            grow, sign, s->nz, b0, v, ldv, out);
+        k_slack_jtv<<<dim3((s->nz + 1023) / 1024, nB), 256, 0, (cudaStream_t)bt->stream>>>(
+            (const unsigned *)s->d_int + 2 * (s->used.size() + 1), s->nz, b0, v, ldv, out);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
