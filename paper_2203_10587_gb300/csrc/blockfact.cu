@@ -117,10 +117,25 @@ __device__ __forceinline__ void invert(const double *D, double *inv, int *neg, i
     *bad = nbad;
 }
 
-// Update phase of one level: targets [t0, t0 + gridDim.x).
+// A column's pivot block D is final: its inverse goes to the diagonal position of L, and its
+// negative and near-zero pivots are counted.
+template <int BS>
+__device__ __forceinline__ void finish_pivot(double *L, int p, int B, int b, const double *D, int *neg,
+                                             int *bad, double tiny) {
+    double Di[BS * BS];
+    int nn, nbad;
+    invert<BS>(D, Di, &nn, &nbad, tiny);
+    store_blk<BS>(L, p, B, b, Di);
+    if (nn) atomicAdd(neg + b, nn);
+    if (nbad) atomicAdd(bad + b, nbad);
+}
+
+// Update phase of one level: targets [t0, t0 + gridDim.x); the diagonal ones also invert their
+// pivot block.
 template <int BS, bool SYM>
 __global__ void __launch_bounds__(kNT) k_bf_update(const DevSymK S, int B, double *T, double *TU,
-                                                   const double *L, const double *U, int t0) {
+                                                   double *L, const double *U, int *neg, int *bad,
+                                                   double tiny, int t0) {
     constexpr int BB = BS * BS;
     const int b = blockIdx.y * kNT + threadIdx.x;
     if (b >= B) return;
@@ -128,7 +143,7 @@ __global__ void __launch_bounds__(kNT) k_bf_update(const DevSymK S, int B, doubl
     const int p = __ldg(S.tgt_blk + t);
     const bool diag = p == __ldg(S.tgt_diag + t);
     const int64_t q0 = __ldg(S.tptr + t), q1 = __ldg(S.tptr + t + 1);
-    if (q0 == q1) return;   // nothing to subtract: T already holds A_IJ
+    if (q0 == q1 && !diag) return;   // nothing to subtract: T already holds A_IJ
     double acc[BB], accU[BB];
     load_blk_cg<BS>(T, p, B, b, acc);
     if (!SYM && !diag) load_blk_cg<BS>(TU, p, B, b, accU);
@@ -150,31 +165,24 @@ __global__ void __launch_bounds__(kNT) k_bf_update(const DevSymK S, int B, doubl
             }
         }
     }
-    store_blk<BS>(T, p, B, b, acc);
+    if (q0 != q1) store_blk<BS>(T, p, B, b, acc);
     if (!SYM && !diag) store_blk<BS>(TU, p, B, b, accU);
+    if (diag) finish_pivot<BS>(L, p, B, b, acc, neg, bad, tiny);
 }
 
-// Scale phase of one level.
+// Scale phase of one level.  (Every target used to invert its column's pivot block for itself: 150
+// FP64 instructions beside the 64 of its product; 2,000 buses x 512: 1.2 ms of the factorisation.)
 template <int BS, bool SYM>
 __global__ void __launch_bounds__(kNT) k_bf_scale(const DevSymK S, int B, const double *T,
-                                                  const double *TU, double *L, double *U,
-                                                  int *neg, int *bad, double tiny, int t0) {
+                                                  const double *TU, double *L, double *U, int t0) {
     constexpr int BB = BS * BS;
     const int b = blockIdx.y * kNT + threadIdx.x;
     if (b >= B) return;
     const int t = t0 + blockIdx.x;
     const int p = __ldg(S.tgt_blk + t), pd = __ldg(S.tgt_diag + t);
-    double D[BB], Di[BB];
-    load_blk_cg<BS>(T, pd, B, b, D);
-    int nn, nbad;
-    invert<BS>(D, Di, &nn, &nbad, tiny);
-    if (p == pd) {
-        store_blk<BS>(L, p, B, b, Di);
-        if (nn) atomicAdd(neg + b, nn);
-        if (nbad) atomicAdd(bad + b, nbad);
-        return;
-    }
-    double X[BB], Y[BB];
+    if (p == pd) return;
+    double Di[BB], X[BB], Y[BB];
+    load_blk_cg<BS>(L, pd, B, b, Di);
     load_blk_cg<BS>(T, p, B, b, X);
     mul<BS>(X, Di, Y);                                          // L_IJ = T_IJ D_J^-1
     store_blk<BS>(L, p, B, b, Y);
@@ -185,20 +193,20 @@ __global__ void __launch_bounds__(kNT) k_bf_scale(const DevSymK S, int B, const 
     }
 }
 
-// ---- split variants: the terms of one target (or one column's sweep) divided among kSlices
-// (kSweepSlices) warps of a block that holds 32 states; slice w takes every kSlices-th term from
-// the w-th, and
-// warp 0 adds the slices' partial sums in slice order.  Used where a level has few targets, so
-// that the long sums of the dense top of the elimination tree are not one thread's latency
-// chain.  The split is fixed by the structure alone (never by the batch size), so every state's
-// result is the same whatever the batch it belongs to.
+// ---- split variants: the terms of one target (or one column's sweep) divided among kSlices warps of
+// a block that holds 32 states; slice w takes every kSlices-th term from the w-th, and the slices'
+// partial sums are added in slice order, an entry or two per warp (one warp alone would be at it
+// longer than at its terms: an FP64 instruction holds its pipe for 64 cycles).  Used where a level
+// has few targets and long sums, so that these are not one thread's latency chain.  The split is
+// fixed by the structure alone (never by the batch size), so every state's result is the same
+// whatever the batch it belongs to.
 constexpr int kSlices = 8;
-constexpr int kSweepSlices = 32;   // the sweeps carry less per term, so they split wider
 
 template <int BS, bool SYM>
 __global__ void __launch_bounds__(32 * kSlices) k_bf_update_split(const DevSymK S, int B, double *T,
-                                                                  double *TU, const double *L,
-                                                                  const double *U, int t0) {
+                                                                  double *TU, double *L,
+                                                                  const double *U, int *neg, int *bad,
+                                                                  double tiny, int t0) {
     constexpr int BB = BS * BS, NP = SYM ? BB : 2 * BB;   // partial sums: lower (and upper)
     __shared__ double part[kSlices][NP][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -208,7 +216,7 @@ __global__ void __launch_bounds__(32 * kSlices) k_bf_update_split(const DevSymK 
     const int p = __ldg(S.tgt_blk + t);
     const bool diag = p == __ldg(S.tgt_diag + t);
     const int64_t q0 = __ldg(S.tptr + t), q1 = __ldg(S.tptr + t + 1);
-    if (q0 == q1) return;   // uniform over the block
+    if (q0 == q1 && !diag) return;   // uniform over the block
     double acc[BB], accU[BB];
 #pragma unroll
     for (int e = 0; e < BB; e++) { acc[e] = 0.0; accU[e] = 0.0; }
@@ -237,34 +245,34 @@ __global__ void __launch_bounds__(32 * kSlices) k_bf_update_split(const DevSymK 
         if (!SYM) part[w][(NP - BB) + e][lane] = accU[e];
     }
     __syncthreads();
+    for (int e = w; e < NP; e += kSlices) {
+        double s = part[0][e][lane];
+#pragma unroll
+        for (int v = 1; v < kSlices; v++) s += part[v][e][lane];
+        part[0][e][lane] = s;   // entry e is this warp's alone
+    }
+    __syncthreads();
     if (w != 0 || !live) return;
     load_blk_cg<BS>(T, p, B, b, acc);
     if (!SYM && !diag) load_blk_cg<BS>(TU, p, B, b, accU);
 #pragma unroll
     for (int e = 0; e < BB; e++) {
-        double s = part[0][e][lane];
-#pragma unroll
-        for (int v = 1; v < kSlices; v++) s += part[v][e][lane];
-        acc[e] += s;
-        if (!SYM) {
-            double su = part[0][(NP - BB) + e][lane];
-#pragma unroll
-            for (int v = 1; v < kSlices; v++) su += part[v][(NP - BB) + e][lane];
-            accU[e] += su;
-        }
+        acc[e] += part[0][e][lane];
+        if (!SYM) accU[e] += part[0][(NP - BB) + e][lane];
     }
-    store_blk<BS>(T, p, B, b, acc);
+    if (q0 != q1) store_blk<BS>(T, p, B, b, acc);
     if (!SYM && !diag) store_blk<BS>(TU, p, B, b, accU);
+    if (diag) finish_pivot<BS>(L, p, B, b, acc, neg, bad, tiny);
 }
 
 // Forward sweep of one level's columns, split: y_J = r_J + (the slices' sums of -F_JK z_K);
 // z_J = D_J^-1 y_J.
 template <int BS>
-__global__ void __launch_bounds__(32 * kSweepSlices) k_bf_forward_split(const DevSymK S, int B,
+__global__ void __launch_bounds__(32 * kSlices) k_bf_forward_split(const DevSymK S, int B,
                                                                    const double *T,
                                                                    const double *L, double *x,
                                                                    int c0) {
-    __shared__ double part[kSweepSlices][BS][32];
+    __shared__ double part[kSlices][BS][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int b = blockIdx.y * 32 + lane;
     const bool live = b < B;
@@ -274,7 +282,7 @@ __global__ void __launch_bounds__(32 * kSweepSlices) k_bf_forward_split(const De
     for (int i = 0; i < BS; i++) y[i] = 0.0;
     const int64_t r0 = __ldg(S.rowptr + J), r1 = __ldg(S.rowptr + J + 1);
     if (live)
-        for (int64_t r = r0 + w; r < r1; r += kSweepSlices) {
+        for (int64_t r = r0 + w; r < r1; r += kSlices) {
             const int K = __ldg(S.rowcol + r), p = __ldg(S.rowblk + r);
             if (!EXAGO_DCHECK(S, K >= 0 && K < S.nb && p >= 0 && p < S.nblk)) continue;
             double F[BS * BS], z[BS];
@@ -289,14 +297,16 @@ __global__ void __launch_bounds__(32 * kSweepSlices) k_bf_forward_split(const De
 #pragma unroll
     for (int i = 0; i < BS; i++) part[w][i][lane] = y[i];
     __syncthreads();
+    if (w < BS && live) {
+        double s = part[0][w][lane];
+#pragma unroll
+        for (int v = 1; v < kSlices; v++) s += part[v][w][lane];
+        part[0][w][lane] = __ldcg(x + ((size_t)J * BS + w) * B + b) + s;
+    }
+    __syncthreads();
     if (w != 0 || !live) return;
 #pragma unroll
-    for (int i = 0; i < BS; i++) {
-        double s = part[0][i][lane];
-#pragma unroll
-        for (int v = 1; v < kSweepSlices; v++) s += part[v][i][lane];
-        y[i] = __ldcg(x + ((size_t)J * BS + i) * B + b) + s;
-    }
+    for (int i = 0; i < BS; i++) y[i] = part[0][i][lane];
     double Di[BS * BS];
     load_blk<BS>(L, __ldg(S.colptr + J), B, b, Di);
 #pragma unroll
@@ -310,11 +320,11 @@ __global__ void __launch_bounds__(32 * kSweepSlices) k_bf_forward_split(const De
 
 // Backward sweep of one level's columns, split: x_J = z_J + (the slices' sums of -U_JI x_I).
 template <int BS, bool SYM>
-__global__ void __launch_bounds__(32 * kSweepSlices) k_bf_backward_split(const DevSymK S, int B,
+__global__ void __launch_bounds__(32 * kSlices) k_bf_backward_split(const DevSymK S, int B,
                                                                     const double *L,
                                                                     const double *U, double *x,
                                                                     int c0) {
-    __shared__ double part[kSweepSlices][BS][32];
+    __shared__ double part[kSlices][BS][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int b = blockIdx.y * 32 + lane;
     const bool live = b < B;
@@ -324,7 +334,7 @@ __global__ void __launch_bounds__(32 * kSweepSlices) k_bf_backward_split(const D
     for (int i = 0; i < BS; i++) v[i] = 0.0;
     const int64_t p0 = __ldg(S.colptr + J), p1 = __ldg(S.colptr + J + 1);
     if (live)
-        for (int64_t p = p0 + 1 + w; p < p1; p += kSweepSlices) {
+        for (int64_t p = p0 + 1 + w; p < p1; p += kSlices) {
             const int I = __ldg(S.rowidx + p);
             if (!EXAGO_DCHECK(S, I >= 0 && I < S.nb)) continue;
             double M[BS * BS], xi[BS];
@@ -340,14 +350,11 @@ __global__ void __launch_bounds__(32 * kSweepSlices) k_bf_backward_split(const D
 #pragma unroll
     for (int i = 0; i < BS; i++) part[w][i][lane] = v[i];
     __syncthreads();
-    if (w != 0 || !live) return;
+    if (w >= BS || !live) return;
+    double s = part[0][w][lane];
 #pragma unroll
-    for (int i = 0; i < BS; i++) {
-        double s = part[0][i][lane];
-#pragma unroll
-        for (int u = 1; u < kSweepSlices; u++) s += part[u][i][lane];
-        x[((size_t)J * BS + i) * B + b] = __ldcg(x + ((size_t)J * BS + i) * B + b) + s;
-    }
+    for (int u = 1; u < kSlices; u++) s += part[u][w][lane];
+    x[((size_t)J * BS + w) * B + b] = __ldcg(x + ((size_t)J * BS + w) * B + b) + s;
 }
 
 // Forward sweep of one level's columns: y_J = r_J - sum_K F_JK z_K; z_J = D_J^-1 y_J.
@@ -506,9 +513,10 @@ __global__ void __launch_bounds__(kNT) k_bf_tail_rhs(const DevSymK S, int B, con
 
 }  // namespace
 
-// A level is split when it has fewer than this many targets (factor) or columns (sweeps): a
-// property of the structure, not of the batch.
-constexpr int kSplitBelow = 64;
+// A level is split when it has fewer than kSplitBelow targets (factor) or columns (sweeps) and a sum of
+// more than kSplitTerms terms: properties of the structure, not of the batch.  Levels of short sums
+// were split too: 200 buses x 37 states spent 200 us in 12 sweep launches of a few terms each.
+constexpr int kSplitBelow = 64, kSplitTerms = 6;
 
 template <int BS, bool SYM>
 int launch_block_factor(const DevSym &S, int B, double *T, double *TU, double *L, double *U,
@@ -519,12 +527,13 @@ int launch_block_factor(const DevSym &S, int B, double *T, double *TU, double *L
         const int t0 = S.lvl_tptr[l], nt = S.sp_tgts[l];
         if (nt <= 0) continue;
         const dim3 grid((unsigned)nt, gy);
-        if (nt < kSplitBelow)
+        if (nt < kSplitBelow && S.sp_pairs[l] > kSplitTerms)
             k_bf_update_split<BS, SYM><<<dim3((unsigned)nt, gy32), 32 * kSlices, 0, st>>>(
-                S.k, B, T, TU, L, U, t0);
+                S.k, B, T, TU, L, U, neg, bad, tiny, t0);
         else
-            k_bf_update<BS, SYM><<<grid, kNT, 0, st>>>(S.k, B, T, TU, L, U, t0);
-        k_bf_scale<BS, SYM><<<grid, kNT, 0, st>>>(S.k, B, T, TU, L, U, neg, bad, tiny, t0);
+            k_bf_update<BS, SYM><<<grid, kNT, 0, st>>>(S.k, B, T, TU, L, U, neg, bad, tiny, t0);
+        if (nt > S.sp_cols[l])   // blocks below a diagonal
+            k_bf_scale<BS, SYM><<<grid, kNT, 0, st>>>(S.k, B, T, TU, L, U, t0);
     }
     if (S.k.tail_n > 0) {
         const int n = S.k.tail_n, R = S.k.nb - S.k.k0, nreal = R * BS;
@@ -552,8 +561,8 @@ int launch_block_solve(const DevSym &S, int B, const double *T, const double *L,
     for (int l = 0; l < S.nlevels; l++) {
         const int c0 = S.lvl_colptr[l], nc = S.sp_cols[l];
         if (nc <= 0) continue;
-        if (nc < kSplitBelow)
-            k_bf_forward_split<BS><<<dim3((unsigned)nc, gy32), 32 * kSweepSlices, 0, st>>>(
+        if (nc < kSplitBelow && S.sp_rows[l] > kSplitTerms)
+            k_bf_forward_split<BS><<<dim3((unsigned)nc, gy32), 32 * kSlices, 0, st>>>(
                 S.k, B, T, L, x, c0);
         else
             k_bf_forward<BS><<<dim3((unsigned)nc, gy), kNT, 0, st>>>(S.k, B, T, L, x, c0);
@@ -568,8 +577,8 @@ int launch_block_solve(const DevSym &S, int B, const double *T, const double *L,
     for (int l = S.nlevels - 1; l >= 0; l--) {
         const int c0 = S.lvl_colptr[l], nc = S.sp_cols[l];
         if (nc <= 0) continue;
-        if (nc < kSplitBelow)
-            k_bf_backward_split<BS, SYM><<<dim3((unsigned)nc, gy32), 32 * kSweepSlices, 0, st>>>(
+        if (nc < kSplitBelow && S.sp_colblks[l] > kSplitTerms)
+            k_bf_backward_split<BS, SYM><<<dim3((unsigned)nc, gy32), 32 * kSlices, 0, st>>>(
                 S.k, B, L, U, x, c0);
         else
             k_bf_backward<BS, SYM><<<dim3((unsigned)nc, gy), kNT, 0, st>>>(S.k, B, L, U, x, c0);
@@ -588,6 +597,9 @@ int upload_block_sym(const BlockSym &S, DevSym &D, std::vector<void *> &allocs) 
     D.lvl_tptr = S.lvl_tptr;
     D.sp_cols = S.sp_cols;
     D.sp_tgts = S.sp_tgts;
+    D.sp_pairs = S.sp_pairs;
+    D.sp_rows = S.sp_rows;
+    D.sp_colblks = S.sp_colblks;
     D.sparse_blocks = S.colptr[S.k0];
     D.k.k0 = S.k0;
     D.k.tail_n = S.tail_n;

@@ -59,7 +59,9 @@ struct BlockSym {
     // pairs with K < k0; tail_r1 [nb]: end of each row's blocks with K < k0; tail_tgt: the target
     // of each lower block (I, J) of the tail, row after row, or -1 where the factor has none.
     int k0 = 0, tail_n = 0;          // first tail column; padded scalar size
-    std::vector<int> sp_cols, sp_tgts, tail_tgt;
+    // sp_pairs, sp_rows, sp_colblks [nlevels]: the most pairs of a target, blocks (J, K) of a row and
+    // blocks (I, J) of a column among the level's columns below k0.
+    std::vector<int> sp_cols, sp_tgts, sp_pairs, sp_rows, sp_colblks, tail_tgt;
     std::vector<int64_t> tail_q1, tail_r1;
     // solve schedule: for each column, in the level order of lvl_cols
     double flops_factor_per_block = 0;   // sum over pairs of one block product (BS^3 FMA units)
@@ -96,7 +98,7 @@ struct DevSymK {
 struct DevSym {
     DevSymK k{};
     int nlevels = 0;
-    std::vector<int> lvl_colptr, lvl_tptr, sp_cols, sp_tgts;
+    std::vector<int> lvl_colptr, lvl_tptr, sp_cols, sp_tgts, sp_pairs, sp_rows, sp_colblks;
     int64_t sparse_blocks = 0;   // factor blocks of the columns before the tail
 };
 

@@ -31,6 +31,24 @@ void merge_without(const std::vector<int> &a, const std::vector<int> &b, int x, 
     }
 }
 
+// The levels' columns, targets and longest sums below k0.
+void sparse_levels(BlockSym &S) {
+    S.sp_cols.assign(S.nlevels, 0);
+    S.sp_tgts = S.sp_pairs = S.sp_rows = S.sp_colblks = S.sp_cols;
+    for (int l = 0; l < S.nlevels; l++) {
+        for (int c = S.lvl_colptr[l]; c < S.lvl_colptr[l + 1]; c++) {
+            const int k = S.lvl_cols[c];
+            if (k >= S.k0) break;   // ascending within a level: the columns below k0 come first
+            S.sp_cols[l]++;
+            S.sp_tgts[l] += (int)(S.colptr[k + 1] - S.colptr[k]);
+            S.sp_rows[l] = std::max(S.sp_rows[l], (int)(S.rowptr[k + 1] - S.rowptr[k]));
+            S.sp_colblks[l] = std::max(S.sp_colblks[l], (int)(S.colptr[k + 1] - S.colptr[k]) - 1);
+        }
+        for (int t = S.lvl_tptr[l]; t < S.lvl_tptr[l] + S.sp_tgts[l]; t++)
+            S.sp_pairs[l] = std::max(S.sp_pairs[l], (int)(S.tptr[t + 1] - S.tptr[t]));
+    }
+}
+
 }  // namespace
 
 bool build_block_sym(int nb, const int *adj_ptr, const int *adj, BlockSym &S, std::string &err) {
@@ -180,12 +198,7 @@ bool build_block_sym(int nb, const int *adj_ptr, const int *adj, BlockSym &S, st
     }
     S.flops_factor_per_block = (double)S.pairs.size();
     S.k0 = nb;
-    S.sp_cols.resize(S.nlevels);
-    S.sp_tgts.resize(S.nlevels);
-    for (int l = 0; l < S.nlevels; l++) {
-        S.sp_cols[l] = S.lvl_colptr[l + 1] - S.lvl_colptr[l];
-        S.sp_tgts[l] = S.lvl_tptr[l + 1] - S.lvl_tptr[l];
-    }
+    sparse_levels(S);
     return true;
 }
 
@@ -221,15 +234,7 @@ void choose_tail(BlockSym &S, int BS, bool sym) {
     const int k0 = best_k0, R = nb - k0;
     S.k0 = k0;
     S.tail_n = best_n;
-    for (int l = 0; l < S.nlevels; l++) {
-        S.sp_cols[l] = S.sp_tgts[l] = 0;
-        for (int c = S.lvl_colptr[l]; c < S.lvl_colptr[l + 1]; c++) {
-            const int k = S.lvl_cols[c];
-            if (k >= k0) continue;   // ascending within a level: the columns below k0 come first
-            S.sp_cols[l]++;
-            S.sp_tgts[l] += (int)(S.colptr[k + 1] - S.colptr[k]);
-        }
-    }
+    sparse_levels(S);
     std::vector<int> col_of_blk(S.nblk);
     for (int k = 0; k < nb; k++)
         for (int64_t p = S.colptr[k]; p < S.colptr[k + 1]; p++) col_of_blk[p] = k;

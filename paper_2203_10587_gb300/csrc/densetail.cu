@@ -502,13 +502,30 @@ __device__ __forceinline__ unsigned long long mag(double v) {
     return u > 0x7ff0000000000000ull ? 0 : u;
 }
 
+__device__ __noinline__ double reciprocal_any(double d) { return 1.0 / d; }
+
+// 1 / d.  The hardware's approximation r0 (rcp.approx.ftz.f64, about 20 bits) and one step of the
+// third-order Householder iteration, r0 + r0 (e + e^2) with e = 1 - d r0: three dependent FP64
+// instructions on the chain of the 64 pivots, in place of the division's ten or so.  Zero,
+// subnormal, huge and non-finite d, where r0 or e would not be ordinary, are divided.
+__device__ __forceinline__ double reciprocal(double d) {
+    const unsigned f = ((unsigned)__double2hiint(d) >> 20) & 0x7ff;
+    if (f - 64u > 1900u) return reciprocal_any(d);
+    double r0;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
+    const double e = fma(-d, r0, 1.0);
+    return fma(r0, fma(e, e, e), r0);
+}
+
 // L D L' (or L D U) of the panel's 64 x 64 diagonal block without pivoting, one block per state;
 // then the inverses of L (and of U'), as digits for the rows below and in FP64, in place of the
 // block, for the sweeps.  Warp w holds columns w, w + 8, .. in registers, a lane rows lane and
-// lane + 32; a step publishes one column.  Bound by the FP64 pipe (about 5,000 warp instructions
-// of 76 cycles over the SM's four) and, alone, by the 64 steps' reciprocals and barriers.
+// lane + 32.  Step k subtracts column k's part from the columns after it; the warp that holds column
+// k + 1 does that one first, and its pivot, reciprocal and publication, while the others work.
+// Bound by the FP64 pipe (about 5,000 warp instructions of 64 cycles over the SM's four) and, for
+// few states, by the chain of pivots: TIMES.
 template <bool SYM, int BS>
-__global__ void __launch_bounds__(kFacThreads) k_dt_factor(int n, int J, double *D, double *V,
+__global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 2) k_dt_factor(int n, int J, double *D, double *V,
                                                            size_t dstride, double *dinv, char *linv,
                                                            int *line, char *uinv, int *uine,
                                                            int *neg, int *bad, double tiny) {
@@ -532,54 +549,66 @@ __global__ void __launch_bounds__(kFacThreads) k_dt_factor(int n, int J, double 
     auto block_max = [&](int c, int j) {
         const int b0 = j / BS * BS;
         const double v = b0 < 32 ? lo[c] : hi[c];
-        unsigned long long a = (lane & ~(BS - 1)) == (b0 & 31) ? mag(v) : 0;
-        for (int h = 16; h > 0; h >>= 1) a = max(a, __shfl_xor_sync(0xffffffffu, a, h));
-        if (lane == 0) s_max[j] = a;
+        if ((lane & ~(BS - 1)) == (b0 & 31)) atomicMax(s_max + j, mag(v));
     };
+    // column k = warp + 8 c is final: its pivot, and the column for the other warps
+    auto publish = [&](int c, int k) {
+        const double d = __shfl_sync(0xffffffffu, c < 4 ? lo[c] : hi[c], k & 31);
+        const double r = reciprocal(d);
+        const double fl = lane > k ? lo[c] : 0.0, fh = lane + 32 > k ? hi[c] : 0.0;
+        s_f[k & 1][lane] = fl;
+        s_f[k & 1][lane + 32] = fh;
+        Ls[k * kPitch + lane] = lane > k ? fl * r : 0.0;
+        Ls[k * kPitch + lane + 32] = lane + 32 > k ? fh * r : 0.0;
+        if (lane == 0) {
+            s_d[k] = d;
+            s_r[k] = r;
+        }
+    };
+    if (tid < 64) s_max[tid] = 0;
+    __syncthreads();
     if (warp < BS) block_max(0, warp);
+    if (warp == 0) publish(0, 0);
 #pragma unroll
     for (int c = 0; c < 8; c++) {
+#pragma unroll 1
         for (int w = 0; w < 8; w++) {
             const int k = 8 * c + w;
-            if (warp == w) {
-                const double d = __shfl_sync(0xffffffffu, c < 4 ? lo[c] : hi[c], k & 31);
-                const double r = 1.0 / d;
-                const double fl = lane > k ? lo[c] : 0.0, fh = lane + 32 > k ? hi[c] : 0.0;
-                s_f[k & 1][lane] = fl;
-                s_f[k & 1][lane + 32] = fh;
-                Ls[k * kPitch + lane] = lane > k ? fl * r : 0.0;
-                Ls[k * kPitch + lane + 32] = lane + 32 > k ? fh * r : 0.0;
-                if (lane == 0) {
-                    s_d[k] = d;
-                    s_r[k] = r;
-                }
-            }
             __syncthreads();
             const double fl = s_f[k & 1][lane], fh = s_f[k & 1][lane + 32];
             const double r = SYM ? 0.0 : s_r[k];
-#pragma unroll
-            for (int q = c; q < 8; q++) {
+            auto update = [&](int q) {   // column warp + 8 q > k loses column k's part
                 const int j = warp + 8 * q;
-                if (j > k) {
-                    double u;
-                    if (SYM) {
-                        u = Ls[k * kPitch + j];
-                    } else {
-                        u = __shfl_sync(0xffffffffu, c < 4 ? lo[q] : hi[q], k & 31) * r;
-                        if (lane == 0) Us[k * kPitch + j] = u;
-                    }
-                    if (c < 4 && (!SYM || q < 4)) lo[q] = fma(-fl, u, lo[q]);
-                    hi[q] = fma(-fh, u, hi[q]);
-                    // column j's block is the next to be eliminated
-                    if ((k + 1) % BS == 0 && j <= k + BS) block_max(q, j);
-                } else if (!SYM && lane == 0) {
-                    Us[k * kPitch + j] = 0.0;
+                double u;
+                if (SYM) {
+                    u = Ls[k * kPitch + j];
+                } else {
+                    u = __shfl_sync(0xffffffffu, c < 4 ? lo[q] : hi[q], k & 31) * r;
+                    if (lane == 0) Us[k * kPitch + j] = u;
                 }
+                if (c < 4 && (!SYM || q < 4)) lo[q] = fma(-fl, u, lo[q]);
+                hi[q] = fma(-fh, u, hi[q]);
+                // column j's block is the next to be eliminated
+                if ((k + 1) % BS == 0 && j <= k + BS) block_max(q, j);
+            };
+            if (w < 7) {
+                if (warp == w + 1) {
+                    update(c);
+                    publish(c, k + 1);
+                } else if (warp > w) {
+                    update(c);
+                }
+            } else if (c < 7 && warp == 0) {
+                update(c + 1 < 8 ? c + 1 : 7);
+                publish(c + 1 < 8 ? c + 1 : 7, k + 1);
             }
+#pragma unroll
+            for (int q = c + 1; q < 8; q++)
+                if (q > c + 1 || w < 7 || warp > 0) update(q);
             if (!SYM)
 #pragma unroll
-                for (int q = 0; q < c; q++)
-                    if (lane == 0) Us[k * kPitch + warp + 8 * q] = 0.0;
+                for (int q = 0; q <= c; q++)
+                    if (lane == 0 && warp + 8 * q <= k) Us[k * kPitch + warp + 8 * q] = 0.0;
         }
     }
     __syncthreads();
