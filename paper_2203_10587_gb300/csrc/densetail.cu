@@ -13,7 +13,8 @@ constexpr int kDigits = 7;            // base-512 digits of a value
 constexpr int kTile = 8192;           // bytes of 64 rows x 64 digits (bf16)
 constexpr int kFlag = 1 << 20;        // row exponent of a row that holds an infinity or a NaN
 constexpr uint32_t kTmemCols = 512;   // 7 sums x 64 columns, allocated as a power of two
-constexpr int kEpi = 256;             // threads that finish products (one row, 32 columns each)
+constexpr int kCols = 16;             // columns of a thread that finishes products (and one row)
+constexpr int kEpi = 128 * (64 / kCols);   // such threads
 constexpr int kUpdThreads = kEpi + 32;
 constexpr int kSmemA = kDigits * 2 * kTile, kSmemB = kDigits * kTile;
 constexpr int kSmemUpd = kSmemA + kSmemB + 1024;   // + alignment of the tiles to 1 KB
@@ -45,25 +46,28 @@ __device__ __forceinline__ long long fixed62(double v, int E) {
 }
 
 // The seven digits of eight neighbouring values of one row, packed as bf16 pairs: out[s] holds
-// the eight digits of weight 512^(6 - s).
+// the eight digits of weight 512^(6 - s).  Adding 256 in each of the six lower places makes every
+// digit a bit field less 256; a digit as a float (2^23 + field, less 2^23 + 256) is exact in bf16, its
+// upper half.
 __device__ __forceinline__ void digits8(const double *v, int E, uint4 *out) {
+    constexpr unsigned long long kHalf =   // 256 (1 + 512 + .. + 512^5)
+        256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36) + (1ull << 45));
     uint32_t p[kDigits][4];
 #pragma unroll
     for (int h = 0; h < 4; h++) {
-        long long X0 = fixed62(v[2 * h], E), X1 = fixed62(v[2 * h + 1], E);
+        uint32_t f[2][kDigits];
 #pragma unroll
-        for (int s = kDigits - 1; s >= 1; s--) {   // lowest digit first: remainder in [-256, 255]
-            X0 += 256;
-            X1 += 256;
-            const float d0 = __uint_as_float(0x4b000000u | ((uint32_t)X0 & 511)) - 8388864.0f;
-            const float d1 = __uint_as_float(0x4b000000u | ((uint32_t)X1 & 511)) - 8388864.0f;
-            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[s][h]) : "f"(d1), "f"(d0));
-            X0 >>= 9;
-            X1 >>= 9;
+        for (int e = 0; e < 2; e++) {
+            const unsigned long long X = (unsigned long long)fixed62(v[2 * h + e], E) + kHalf;
+            const uint32_t lo = (uint32_t)X, hi = (uint32_t)(X >> 32);
+            const uint32_t d[kDigits] = {0, hi >> 13, hi >> 4, __funnelshift_r(lo, hi, 27), lo >> 18, lo >> 9, lo};
+#pragma unroll
+            for (int s = 1; s < kDigits; s++)
+                f[e][s] = __float_as_uint(__uint_as_float((d[s] & 511) | 0x4b000000u) - 8388864.0f);
+            f[e][0] = __float_as_uint(__uint_as_float(0x4b000000u + (uint32_t)(((int)hi >> 22) + 512)) - 8389120.0f);
         }
-        const float t0 = __uint_as_float(0x4b000000u + (uint32_t)((int)X0 + 512)) - 8389120.0f;
-        const float t1 = __uint_as_float(0x4b000000u + (uint32_t)((int)X1 + 512)) - 8389120.0f;
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[0][h]) : "f"(t1), "f"(t0));
+#pragma unroll
+        for (int s = 0; s < kDigits; s++) p[s][h] = __byte_perm(f[0][s], f[1][s], 0x7632);
     }
 #pragma unroll
     for (int s = 0; s < kDigits; s++) out[s] = make_uint4(p[s][0], p[s][1], p[s][2], p[s][3]);
@@ -222,27 +226,27 @@ __device__ __forceinline__ void tmem_sums4(uint32_t addr, float (*v)[4]) {
 #pragma unroll
         for (int c = 0; c < 4; c++) v[g][c] = __uint_as_float(r[g][c]);
 }
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpi) : "memory"); }
 
-// The thread's 32 values, eight places on: the loops below take eight values at a time from the
-// front, so that their bodies are in the instruction cache once (unrolled over all 32 columns, half
-// of the stalls were for instructions).
+// The thread's values, eight places on: the loops below take eight values at a time from the front,
+// so that their bodies are in the instruction cache once (unrolled over all columns, half of the
+// stalls were for instructions).
 __device__ __forceinline__ void rotate8(double *v) {
     double t[8];
 #pragma unroll
     for (int i = 0; i < 8; i++) t[i] = v[i];
 #pragma unroll
-    for (int i = 0; i < 24; i++) v[i] = v[i + 8];
+    for (int i = 0; i < kCols - 8; i++) v[i] = v[i + 8];
 #pragma unroll
-    for (int i = 0; i < 8; i++) v[24 + i] = t[i];
+    for (int i = 0; i < 8; i++) v[kCols - 8 + i] = t[i];
 }
 
-// acc[0..31] -= (sub) or = the product in TMEM, this thread's row and 32 columns from c0; ea: the
-// row's exponent, eb [64] the columns' (shared memory).
+// acc[0 .. kCols) -= (sub) or = the product in TMEM, this thread's row and kCols columns from c0; ea:
+// the row's exponent, eb [64] the columns' (shared memory).
 __device__ __forceinline__ void take_product(uint32_t tmem, int c0, int ea, const int *eb, double *acc,
                                              bool sub) {
 #pragma unroll 1
-    for (int q = 0; q < 4; q++) {
+    for (int q = 0; q < kCols / 8; q++) {
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             float d[kDigits][4];
@@ -285,7 +289,7 @@ __device__ __forceinline__ size_t digit_at(int P, int K, int s, int I) {
 // MODE 0: F and L (SYM); 1: F alone (LU, lower side); 2: U' from G = U' D' (LU, upper side).
 // What bounds it: the 28 x 4 tensor instructions of a 64-deep step (128 x 64 x 16 each) and, as
 // much, the 8,192 targets' integer joins and two FP64-pipe instructions each; one block per SM
-// (172 KB of digits), 8 warps that finish products beside one that issues copies and MMAs.
+// (172 KB of digits), 16 warps that finish products beside one that issues copies and MMAs.
 // A wait that gives up sets the status word and the block's flag; the block then runs to its end
 // on whatever it holds, so that every barrier is met.
 template <bool DIAG, int MODE>
@@ -294,7 +298,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
     __shared__ uint64_t bar_full, bar_mma, bar_epi, bar_tgt;
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_dead;
-    __shared__ int s_eb[2][64], s_em[2][128];
+    __shared__ int s_eb[2][64], s_em[64 / kCols][128];
     char *sA = (char *)(((uintptr_t)raw + 1023) & ~(uintptr_t)1023), *sB = sA + kSmemA;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const size_t st = blockIdx.y;
@@ -354,17 +358,17 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
         }
         __syncwarp();
     } else {
-        const int half = warp >> 2;                       // columns 32 half ..
-        const int row = ((warp & 3) << 5) | lane, c0 = 32 * half;
+        const int part = warp >> 2;                       // columns kCols part ..
+        const int row = ((warp & 3) << 5) | lane, c0 = kCols * part;
         const int grow = 64 * I0 + row;                   // row of the matrix
         const bool live = row < 64 * tiles;
         const uint32_t tw = tmem + ((uint32_t)(warp & 3) << 21);
         const int ld = n - 64 * J;
         double *Dp = A.D + st * A.dstride + tail_pos(n, 64 * J, 64 * J) + (size_t)c0 * ld +
                      (grow - 64 * J);
-        double acc[32];
+        double acc[kCols];
 #pragma unroll
-        for (int c = 0; c < 32; c++) acc[c] = live ? __ldcg(Dp + (size_t)c * ld) : 0.0;
+        for (int c = 0; c < kCols; c++) acc[c] = live ? __ldcg(Dp + (size_t)c * ld) : 0.0;
         const int *xa = A.xa + st * (size_t)P * n, *xb = A.xb + st * (size_t)P * n;
         const double *dinv = A.dinv + st * n + 64 * J + c0;
         // steps K < J: the products of the panels before; J: the targets times the inverse, F_IJ
@@ -381,18 +385,19 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
                 if (K == J && tid < 64) s_eb[J & 1][tid] = __ldcg(A.inve + st * 64 + tid);
                 int E = 1;
 #pragma unroll
-                for (int c = 0; c < 32; c++) E = max(E, exp_field(acc[c]));
-                s_em[half][row] = E;
+                for (int c = 0; c < kCols; c++) E = max(E, exp_field(acc[c]));
+                s_em[part][row] = E;
                 epi_sync();
-                E = max(E, s_em[half ^ 1][row]);
+#pragma unroll
+                for (int h = 0; h < 64 / kCols; h++) E = max(E, s_em[h][row]);
                 ea = row_exp(E);
 #pragma unroll 1
-                for (int q = 0; q < 4; q++) {
+                for (int q = 0; q < kCols / 8; q++) {
                     uint4 o[kDigits];
                     digits8(acc, E, o);
 #pragma unroll
                     for (int s = 0; s < kDigits; s++)
-                        *(uint4 *)(sA + s * 2 * kTile + tile_at(row, 4 * half + q)) = o[s];
+                        *(uint4 *)(sA + s * 2 * kTile + tile_at(row, kCols / 8 * part + q)) = o[s];
                     rotate8(acc);
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -408,15 +413,15 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
                 if (!DIAG && K == J) {
                     if (MODE == 2)
 #pragma unroll
-                        for (int c = 0; c < 32; c++) acc[c] *= __ldcg(dinv + c);
+                        for (int c = 0; c < kCols; c++) acc[c] *= __ldcg(dinv + c);
                     if (live)
 #pragma unroll
-                        for (int c = 0; c < 32; c++) Dp[(size_t)c * ld] = acc[c];
+                        for (int c = 0; c < kCols; c++) Dp[(size_t)c * ld] = acc[c];
                 }
             } else {
                 const bool second = K == J + 2;
                 int *xo = (second ? A.yb : A.ya) + st * (size_t)P * n + (size_t)J * n + grow;
-                if (half == 0 && live) *xo = ea;
+                if (part == 0 && live) *xo = ea;
                 epi_sync();
                 if (tid == 0) {
                     char *out = (second ? A.ob : A.oa) + st * A.sstride;
@@ -427,13 +432,13 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
                 }
                 if (MODE == 0 && !second)
 #pragma unroll
-                    for (int c = 0; c < 32; c++) acc[c] *= __ldcg(dinv + c);
+                    for (int c = 0; c < kCols; c++) acc[c] *= __ldcg(dinv + c);
                 epi_sync();
             }
         }
         if (DIAG && live)
 #pragma unroll
-            for (int c = 0; c < 32; c++) Dp[(size_t)c * ld] = acc[c];
+            for (int c = 0; c < kCols; c++) Dp[(size_t)c * ld] = acc[c];
     }
     __syncthreads();
     if (warp == kEpi / 32)
@@ -522,10 +527,10 @@ __device__ __forceinline__ double reciprocal(double d) {
 // block, for the sweeps.  Warp w holds columns w, w + 8, .. in registers, a lane rows lane and
 // lane + 32.  Step k subtracts column k's part from the columns after it; the warp that holds column
 // k + 1 does that one first, and its pivot, reciprocal and publication, while the others work.
-// Bound by the FP64 pipe (about 5,000 warp instructions of 64 cycles over the SM's four) and, for
-// few states, by the chain of pivots: TIMES.
+// Bound by the FP64 pipe (about 5,000 warp instructions of 64 cycles over four pipes) and, for
+// few states, by the chain of pivots: 192 us for 512 states (290 before the look-ahead), 72 for 37.
 template <bool SYM, int BS>
-__global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 2) k_dt_factor(int n, int J, double *D, double *V,
+__global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 3) k_dt_factor(int n, int J, double *D, double *V,
                                                            size_t dstride, double *dinv, char *linv,
                                                            int *line, char *uinv, int *uine,
                                                            int *neg, int *bad, double tiny) {
@@ -575,16 +580,16 @@ __global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 2) k_dt_factor(int n, i
         for (int w = 0; w < 8; w++) {
             const int k = 8 * c + w;
             __syncthreads();
-            const double fl = s_f[k & 1][lane], fh = s_f[k & 1][lane + 32];
-            const double r = SYM ? 0.0 : s_r[k];
+            const double fl = SYM ? s_f[k & 1][lane] : Ls[k * kPitch + lane];
+            const double fh = SYM ? s_f[k & 1][lane + 32] : Ls[k * kPitch + lane + 32];
             auto update = [&](int q) {   // column warp + 8 q > k loses column k's part
                 const int j = warp + 8 * q;
-                double u;
+                double u;   // SYM: F's column times L's row; else L's column times the row of D U
                 if (SYM) {
                     u = Ls[k * kPitch + j];
                 } else {
-                    u = __shfl_sync(0xffffffffu, c < 4 ? lo[q] : hi[q], k & 31) * r;
-                    if (lane == 0) Us[k * kPitch + j] = u;
+                    u = __shfl_sync(0xffffffffu, c < 4 ? lo[q] : hi[q], k & 31);
+                    if (lane == 0) Us[k * kPitch + j] = u;   // D U, scaled at the end
                 }
                 if (c < 4 && (!SYM || q < 4)) lo[q] = fma(-fl, u, lo[q]);
                 hi[q] = fma(-fh, u, hi[q]);
@@ -622,6 +627,10 @@ __global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 2) k_dt_factor(int n, i
             0xffffffffu, !(fabs(d) > tiny * __longlong_as_double((long long)a))));
         if (lane == 0 && nn) atomicAdd(neg + st, nn);
         if (lane == 0 && nb) atomicAdd(bad + st, nb);
+    }
+    if (!SYM) {
+        for (int e = tid; e < 64 * 64; e += kFacThreads) Us[(e >> 6) * kPitch + (e & 63)] *= s_r[e >> 6];
+        __syncthreads();
     }
     for (int side = 0; side < (SYM ? 1 : 2); side++) {
         double *M = side ? Us : Ls;
