@@ -145,8 +145,13 @@ __global__ void __launch_bounds__(kNT) k_bf_update(const DevSymK S, int B, doubl
     const int64_t q0 = __ldg(S.tptr + t), q1 = __ldg(S.tptr + t + 1);
     if (q0 == q1 && !diag) return;   // nothing to subtract: T already holds A_IJ
     double acc[BB], accU[BB];
-    load_blk_cg<BS>(T, p, B, b, acc);
-    if (!SYM && !diag) load_blk_cg<BS>(TU, p, B, b, accU);
+    if (__ldg(S.tgt_fill + t)) {   // A_IJ = 0, not assembled
+#pragma unroll
+        for (int e = 0; e < BB; e++) { acc[e] = 0.0; accU[e] = 0.0; }
+    } else {
+        load_blk_cg<BS>(T, p, B, b, acc);
+        if (!SYM && !diag) load_blk_cg<BS>(TU, p, B, b, accU);
+    }
     for (int64_t q = q0; q < q1; q++) {
         const int2 pr = __ldg(S.pairs + q);   // (I, K), (J, K)
         if (!EXAGO_DCHECK(S, pr.x >= 0 && pr.x < S.nblk && pr.y >= 0 && pr.y < S.nblk)) continue;
@@ -253,8 +258,13 @@ __global__ void __launch_bounds__(32 * kSlices) k_bf_update_split(const DevSymK 
     }
     __syncthreads();
     if (w != 0 || !live) return;
-    load_blk_cg<BS>(T, p, B, b, acc);
-    if (!SYM && !diag) load_blk_cg<BS>(TU, p, B, b, accU);
+    if (__ldg(S.tgt_fill + t)) {
+#pragma unroll
+        for (int e = 0; e < BB; e++) { acc[e] = 0.0; accU[e] = 0.0; }
+    } else {
+        load_blk_cg<BS>(T, p, B, b, acc);
+        if (!SYM && !diag) load_blk_cg<BS>(TU, p, B, b, accU);
+    }
 #pragma unroll
     for (int e = 0; e < BB; e++) {
         acc[e] += part[0][e][lane];
@@ -420,6 +430,17 @@ __global__ void __launch_bounds__(kNT) k_bf_backward(const DevSymK S, int B, con
     for (int i = 0; i < BS; i++) x[((size_t)J * BS + i) * B + b] = v[i];
 }
 
+// BS values v[0], v[step], .. to consecutive, aligned doubles.
+template <int BS>
+__device__ __forceinline__ void store_col(double *p, const double *v, int step) {
+    if constexpr (BS == 4)
+        asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[step]),
+                     "d"(v[2 * step]), "d"(v[3 * step])
+                     : "memory");
+    else
+        *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[step]);
+}
+
 // The tail's panels from the assembled blocks: T_IJ = A_IJ - sum over the columns K < k0 of
 // F_IK U_KJ, one thread per (state, lower block of the tail), written where densetail.h keeps it
 // (LU: the upper block, transposed, into V; inside a 64-column panel's own square also in place).
@@ -442,8 +463,10 @@ __global__ void __launch_bounds__(kNT) k_bf_tail(const DevSymK S, int B, const d
     const int t = __ldg(S.tail_tgt + e);
     if (t >= 0) {
         const int p = __ldg(S.tgt_blk + t);
-        load_blk_cg<BS>(T, p, B, b, acc);
-        if (!SYM) load_blk_cg<BS>(TU, p, B, b, accU);
+        if (!__ldg(S.tgt_fill + t)) {
+            load_blk_cg<BS>(T, p, B, b, acc);
+            if (!SYM) load_blk_cg<BS>(TU, p, B, b, accU);
+        }
         for (int64_t q = __ldg(S.tptr + t), q1 = __ldg(S.tail_q1 + t); q < q1; q++) {
             const int2 pr = __ldg(S.pairs + q);
             if (!EXAGO_DCHECK(S, pr.x >= 0 && pr.x < S.nblk && pr.y >= 0 && pr.y < S.nblk)) continue;
@@ -460,15 +483,17 @@ __global__ void __launch_bounds__(kNT) k_bf_tail(const DevSymK S, int B, const d
     }
     const int n = S.tail_n, r0 = BS * i, c0 = BS * j;
     double *Db = D + (size_t)b * dstride, *Vb = SYM ? nullptr : V + (size_t)b * dstride;
+    // a block's column is BS consecutive rows, aligned (r0 and the panels' heights are multiples of
+    // BS): one store of a whole 16- or 32-byte piece, since the lanes' states lie apart
 #pragma unroll
-    for (int c = 0; c < BS; c++)
-#pragma unroll
-        for (int r = 0; r < BS; r++) {
-            Db[tail_pos(n, r0 + r, c0 + c)] = acc[r * BS + c];
-            if (SYM || i == j) continue;
-            if ((r0 >> 6) == (c0 >> 6)) Db[tail_pos(n, c0 + c, r0 + r)] = accU[c * BS + r];
-            else Vb[tail_pos(n, r0 + r, c0 + c)] = accU[c * BS + r];
-        }
+    for (int c = 0; c < BS; c++) {
+        store_col<BS>(Db + tail_pos(n, r0, c0 + c), acc + c, BS);
+        if (SYM || i == j) continue;
+        if ((r0 >> 6) == (c0 >> 6))   // row c of U_JI's block is column r of the transpose
+            store_col<BS>(Db + tail_pos(n, c0, r0 + c), accU + c, BS);
+        else
+            store_col<BS>(Vb + tail_pos(n, r0, c0 + c), accU + c * BS, 1);
+    }
 }
 
 // Identity in the rows that pad the tail to a multiple of 64: one thread per entry and state.
@@ -619,6 +644,7 @@ int upload_block_sym(const BlockSym &S, DevSym &D, std::vector<void *> &allocs) 
     if (!e) e = up(S.vec.data(), S.vec.size() * sizeof(S.vec[0]), (const void **)&D.k.field)
     UPV(colptr, colptr); UPV(rowidx, rowidx); UPV(rowptr, rowptr); UPV(rowblk, rowblk);
     UPV(rowcol, rowcol); UPV(lvl_cols, lvl_cols); UPV(tgt_blk, tgt_blk); UPV(tgt_diag, tgt_diag);
+    UPV(tgt_fill, tgt_fill);
     UPV(tptr, tptr); UPV(pairs, pairs); UPV(tail_tgt, tail_tgt); UPV(tail_q1, tail_q1);
     UPV(tail_r1, tail_r1);
 #undef UPV

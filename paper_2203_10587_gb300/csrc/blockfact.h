@@ -51,6 +51,8 @@ struct BlockSym {
     std::vector<int> lvl_tptr;       // [nlevels + 1] into targets
     std::vector<int> tgt_blk;        // block position of each target
     std::vector<int> tgt_diag;       // block position of the target column's diagonal
+    std::vector<int> tgt_fill;       // 1: a fill block, zero in A; it always has update pairs
+    std::vector<int> own_blk;        // the blocks of A's own pattern, ascending
     std::vector<int64_t> tptr;       // [ntargets + 1]
     std::vector<int2> pairs;         // (position of (I, K), position of (J, K))
     // dense tail (densetail.h): the columns k0 .. nb - 1 are factored as one dense matrix per
@@ -85,7 +87,7 @@ struct DevSymK {
     const int64_t *rowptr;   // [nb + 1]
     const int *rowblk, *rowcol;
     const int *lvl_cols;     // [nb]
-    const int *tgt_blk, *tgt_diag;
+    const int *tgt_blk, *tgt_diag, *tgt_fill;
     const int64_t *tptr;
     const int2 *pairs;
     int *status;             // the owning net's device status word (debug-build index checks)
@@ -105,8 +107,9 @@ struct DevSym {
 // Uploads S (cudaMalloc through dev_malloc; the pointers go to `allocs` for the owner to free).
 int upload_block_sym(const BlockSym &S, DevSym &D, std::vector<void *> &allocs);
 
-// Batched numeric factorisation and solve on DevSym.  T: the assembled matrix A, lower blocks
-// (and TU the upper blocks, the transposed positions, for LU), [nblk][BS*BS][B]; overwritten by
+// Batched numeric factorisation and solve on DevSym.  T: the assembled matrix A, the lower blocks
+// of its own pattern (own_blk; and TU the upper blocks, the transposed positions, for LU),
+// [nblk][BS*BS][B]; overwritten by
 // F = L D (and U D) in the columns before the tail.  L: [sparse_blocks][BS*BS][B] receives L
 // (off-diagonal) and D^-1 (diagonal positions) of those columns; U likewise for LU.  tail: the
 // workspace of tail_shape(S.k.tail_n, B, SYM), which receives the tail's factor.  neg [B] counts the negative pivots of the diagonal blocks'

@@ -67,6 +67,7 @@ bool build_block_sym(int nb, const int *adj_ptr, const int *adj, BlockSym &S, st
         std::sort(a.begin(), a.end());
         a.erase(std::unique(a.begin(), a.end()), a.end());
     }
+    const std::vector<std::vector<int>> own = g;   // A's pattern
     // minimum degree, lowest index on ties
     std::set<std::pair<int, int>> queue;
     for (int v = 0; v < nb; v++) queue.insert({(int)g[v].size(), v});
@@ -197,6 +198,13 @@ bool build_block_sym(int nb, const int *adj_ptr, const int *adj, BlockSym &S, st
         });
     }
     S.flops_factor_per_block = (double)S.pairs.size();
+    S.tgt_fill.assign(ntgt, 0);
+    for (int k = 0; k < nb; k++)
+        for (int64_t p = S.colptr[k]; p < S.colptr[k + 1]; p++) {
+            const int u = S.perm[S.rowidx[p]], v = S.perm[k];
+            if (u == v || std::binary_search(own[u].begin(), own[u].end(), v)) S.own_blk.push_back((int)p);
+            else S.tgt_fill[tgt_of_blk[p]] = 1;
+        }
     S.k0 = nb;
     sparse_levels(S);
     return true;

@@ -652,7 +652,23 @@ __global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 3) k_dt_factor(int n, i
 
 // ---- sweeps --------------------------------------------------------------------------------------
 
-constexpr int kSolThreads = 256;
+constexpr int kSolThreads = 256;   // eight warps of eight columns
+
+// The warp's sums of a[0 .. 8): lanes 4 c .. 4 c + 3 receive that of a[c].  Half of the values move to
+// the other half of the lanes at each of three steps, so 9 additions in place of 40.
+__device__ __forceinline__ double sum8(double *a, int lane) {
+#pragma unroll
+    for (int h = 4; h >= 1; h >>= 1) {
+        const bool up = lane & (4 * h);
+#pragma unroll
+        for (int c = 0; c < h; c++) {
+            const double give = up ? a[c] : a[c + h], keep = up ? a[c + h] : a[c];
+            a[c] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * h);
+        }
+    }
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+    return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
+}
 
 // Both sweeps of one state's tail.  Forward, per panel: z = L^-1 r, the rows below lose F D^-1 z;
 // backward: the panel's unknowns lose U's (or D^-1 F's) part, then L^-T (U^-1).
@@ -692,19 +708,31 @@ __global__ void __launch_bounds__(kSolThreads) k_dt_solve(int n, int nreal, int 
     for (int J = P - 1; J >= 0; J--) {
         const int ld = n - 64 * J, j0 = 64 * J;
         const double *Vp = Vb + tail_pos(n, j0, j0);
-        for (int c = warp; c < 64; c += kSolThreads / 32) {   // a warp per column
-            double a = 0.0;
-            for (int i = 64 + lane; i < ld; i += 32) a = fma(__ldg(Vp + (size_t)c * ld + i), sx[j0 + i], a);
-            for (int h = 16; h > 0; h >>= 1) a += __shfl_xor_sync(0xffffffffu, a, h);
-            if (lane == 0) part[c] = SYM ? fma(-a, __ldg(di + j0 + c), sx[j0 + c]) : sx[j0 + c] - a;
+        {   // a warp's eight columns together
+            double a[8];
+#pragma unroll
+            for (int c = 0; c < 8; c++) a[c] = 0.0;
+            const double *p = Vp + (size_t)(8 * warp) * ld;
+            for (int i = 64 + lane; i < ld; i += 32) {
+                const double xi = sx[j0 + i];
+#pragma unroll
+                for (int c = 0; c < 8; c++) a[c] = fma(__ldg(p + (size_t)c * ld + i), xi, a[c]);
+            }
+            const double t = sum8(a, lane);
+            const int c = 8 * warp + (lane >> 2);
+            if ((lane & 3) == 0) part[c] = SYM ? fma(-t, __ldg(di + j0 + c), sx[j0 + c]) : sx[j0 + c] - t;
         }
         __syncthreads();
         // x_k = sum_i X[i][k] w_i, X = L^-1 (SYM) or U'^-1: column k of the panel's inverse
-        for (int c = warp; c < 64; c += kSolThreads / 32) {
-            double a = __ldg(Vp + (size_t)c * ld + lane) * part[lane];
-            a = fma(__ldg(Vp + (size_t)c * ld + lane + 32), part[lane + 32], a);
-            for (int h = 16; h > 0; h >>= 1) a += __shfl_xor_sync(0xffffffffu, a, h);
-            if (lane == 0) sx[j0 + c] = a;
+        {
+            double a[8];
+            const double *p = Vp + (size_t)(8 * warp) * ld + lane;
+            const double w0 = part[lane], w1 = part[lane + 32];
+#pragma unroll
+            for (int c = 0; c < 8; c++)
+                a[c] = fma(__ldg(p + (size_t)c * ld + 32), w1, __ldg(p + (size_t)c * ld) * w0);
+            const double t = sum8(a, lane);
+            if ((lane & 3) == 0) sx[j0 + 8 * warp + (lane >> 2)] = t;
         }
         __syncthreads();
     }

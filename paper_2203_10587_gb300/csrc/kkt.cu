@@ -58,15 +58,16 @@ __device__ __forceinline__ const double *hrow(const KktDev &K, const double *jv,
     return jv + K.nnzJg + 4 * ((size_t)side * K.nl + l);
 }
 
-// Assembly of the reduced matrix: one thread per (state, block).
+// Assembly of the reduced matrix: one thread per (state, block of its own pattern).
 __global__ void __launch_bounds__(KNT) k_kkt_assemble(const KktDev K, const DevSymK S, int B,
+                                                      const int *__restrict__ own,
                                                       const double *__restrict__ jval,
                                                       const double *__restrict__ hval,
                                                       const double *__restrict__ dx,
                                                       const double *__restrict__ dc, double *T) {
     const int b = blockIdx.y * KNT + threadIdx.x;
     if (b >= B) return;
-    const int p = blockIdx.x;
+    const int p = __ldg(own + blockIdx.x);
     const double *jv = jval + (size_t)b * K.nnzJ, *hv = hval + (size_t)b * K.nnzH;
     const double *dxb = dx + (size_t)b * K.n, *dcb = dc + (size_t)b * K.m;
     double v[16];
@@ -246,6 +247,7 @@ struct exago_kkt {
     BlockSym S;
     DevSym D;
     KktDev K{};
+    const int *own_blk = nullptr;   // device copy of S.own_blk
     std::vector<void *> allocs;
     std::mutex mu;            // the internal workspace
     void *ws = nullptr;
@@ -400,6 +402,7 @@ exago_status exago_kkt_create(exago_net_t net, exago_kkt_t *out) {
         KktDev &K = k->K;
         K.nb = nb; K.nl = nl; K.ng = ng; K.n = n; K.m = m;
         K.nnzJ = P->nnzJ; K.nnzH = P->nnzH; K.nnzJg = P->nnzJg; K.hpg = P->Hrowptr[2 * nb];
+        if (s == EXAGO_OK) s = upload_vec(k, S.own_blk, &k->own_blk);
         if (s == EXAGO_OK) s = upload_vec(k, asrc, &K.asm_src);
         if (s == EXAGO_OK) s = upload_vec(k, adiag, &K.asm_diag);
         if (s == EXAGO_OK) s = upload_vec(k, S.perm, &K.bus_of_col);
@@ -515,8 +518,8 @@ exago_status exago_kkt_solve(exago_kkt_t kkt, int B, const double *jval, const d
     const unsigned gy = (unsigned)((B + KNT - 1) / KNT);
     cudaError_t e = cudaMemsetAsync(neg, 0, 2 * (size_t)B * sizeof(int), st);
     if (e != cudaSuccess) return set_last_error(EXAGO_ECUDA, cudaGetErrorString(e));
-    k_kkt_assemble<<<dim3((unsigned)kkt->S.nblk, gy), KNT, 0, st>>>(K, kkt->D.k, B, jval, hval, dx,
-                                                                    dc, T);
+    k_kkt_assemble<<<dim3((unsigned)kkt->S.own_blk.size(), gy), KNT, 0, st>>>(
+        K, kkt->D.k, B, kkt->own_blk, jval, hval, dx, dc, T);
     k_kkt_rhs<<<dim3((unsigned)K.nb, gy), KNT, 0, st>>>(K, B, jval, hval, dx, dc, rhs, x, neg);
     int le = launch_block_factor<4, true>(kkt->D, B, T, nullptr, L, nullptr, neg, bad, kTiny, tail, st);
     if (le == 0) le = launch_block_solve<4, true>(kkt->D, B, T, L, nullptr, x, tail, st);

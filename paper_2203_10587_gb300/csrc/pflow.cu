@@ -43,12 +43,13 @@ __device__ __forceinline__ double pf_src(int s, const double *jv) {
     return s >= 0 ? __ldg(jv + s) : s == -2 ? 1.0 : 0.0;
 }
 
-__global__ void __launch_bounds__(PNT) k_pf_assemble(const PfDev P, int B, int64_t nblk,
+__global__ void __launch_bounds__(PNT) k_pf_assemble(const PfDev P, int B,
+                                                     const int *__restrict__ own,
                                                      const double *__restrict__ jval, double *T,
                                                      double *TU) {
     const int b = blockIdx.y * PNT + threadIdx.x;
     if (b >= B) return;
-    const int64_t p = blockIdx.x;
+    const int64_t p = __ldg(own + blockIdx.x);
     const double *jv = jval + (size_t)b * P.nnzJ;
 #pragma unroll
     for (int e = 0; e < 4; e++) {
@@ -101,6 +102,7 @@ size_t r256(size_t v) { return (v + 255) / 256 * 256; }
 using namespace exago;
 
 struct exago_pf {
+    const int *own_blk = nullptr;   // device copy of S.own_blk
     exago_net_t net = nullptr;
     BlockSym S;
     DevSym D;
@@ -229,6 +231,7 @@ exago_status exago_pf_create(exago_net_t net, const int *bus_type, exago_pf_t *o
         PfDev &D = pf->P;
         D.nb = nb; D.n = P->n; D.m = P->m; D.nnzJ = P->nnzJ;
         if (P->nnzJ >= (1ll << 31)) s = set_last_error(EXAGO_EINVAL, "grid too large");
+        if (s == EXAGO_OK) s = pf_upload(pf, S.own_blk, &pf->own_blk);
         if (s == EXAGO_OK) s = pf_upload(pf, lo, &D.src_lo);
         if (s == EXAGO_OK) s = pf_upload(pf, up, &D.src_up);
         if (s == EXAGO_OK) s = pf_upload(pf, S.iperm, &D.col_of_bus);
@@ -320,7 +323,7 @@ exago_status exago_pf_step(exago_pf_t pf, const exago_batch *batch, double *x_ne
     if (e != cudaSuccess) return set_last_error(EXAGO_ECUDA, cudaGetErrorString(e));
     const PfDev &D = pf->P;
     const unsigned gy = (unsigned)((B + PNT - 1) / PNT);
-    k_pf_assemble<<<dim3((unsigned)pf->S.nblk, gy), PNT, 0, st>>>(D, B, pf->S.nblk, jv, T, TU);
+    k_pf_assemble<<<dim3((unsigned)pf->S.own_blk.size(), gy), PNT, 0, st>>>(D, B, pf->own_blk, jv, T, TU);
     k_pf_rhs<<<dim3((unsigned)D.nb, gy), PNT, 0, st>>>(D, B, gh, x, mis);
     int le = launch_block_factor<2, false>(pf->D, B, T, TU, L, U, neg, bad, kPfTiny, tail, st);
     if (le == 0) le = launch_block_solve<2, false>(pf->D, B, T, L, U, x, tail, st);
