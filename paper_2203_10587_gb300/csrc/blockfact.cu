@@ -198,6 +198,85 @@ __global__ void __launch_bounds__(kNT) k_bf_scale(const DevSymK S, int B, const 
     }
 }
 
+// ---- small batches: a block's rows on different warps (threads 32 states x BS rows), so that a
+// block product is 16 dependent-free multiply-adds a warp in place of 64 (an FP64 instruction holds
+// its pipe for 64 cycles whatever the lanes).  Every element's sum is the same, so results do not
+// depend on the choice.
+constexpr int kRowsBelow = 129;   // states
+
+// acc[j] (row r of target t) less its pairs up to q1; accU likewise for the upper block (LU).
+template <int BS, bool SYM>
+__device__ __forceinline__ void row_sums(const DevSymK &S, int B, int b, int r, int64_t q0, int64_t q1,
+                                         const double *T, const double *L, const double *U, bool upper,
+                                         double *acc, double *accU) {
+    constexpr int BB = BS * BS;
+    auto row = [&](const double *A, int64_t p, double *v) {
+#pragma unroll
+        for (int k = 0; k < BS; k++) v[k] = __ldcg(A + ((size_t)p * BB + r * BS + k) * B + b);
+    };
+    for (int64_t q = q0; q < q1; q++) {
+        const int2 pr = __ldg(S.pairs + q);
+        if (!EXAGO_DCHECK(S, pr.x >= 0 && pr.x < S.nblk && pr.y >= 0 && pr.y < S.nblk)) continue;
+        double X[BS], Y[BB];
+        row(T, pr.x, X);
+        load_blk_cg<BS>(SYM ? L : U, pr.y, B, b, Y);
+#pragma unroll
+        for (int j = 0; j < BS; j++)
+#pragma unroll
+            for (int k = 0; k < BS; k++) acc[j] = fma(-X[k], SYM ? Y[j * BS + k] : Y[k * BS + j], acc[j]);
+        if (!SYM && upper) {
+            row(T, pr.y, X);
+            load_blk_cg<BS>(U, pr.x, B, b, Y);
+#pragma unroll
+            for (int j = 0; j < BS; j++)
+#pragma unroll
+                for (int k = 0; k < BS; k++) accU[j] = fma(-X[k], Y[k * BS + j], accU[j]);
+        }
+    }
+}
+
+// Row r of target t's own block (zero for a fill block).
+template <int BS>
+__device__ __forceinline__ void own_row(const DevSymK &S, const double *A, int t, int p, int B, int b, int r,
+                                        double *v) {
+    const bool fill = __ldg(S.tgt_fill + t);
+#pragma unroll
+    for (int k = 0; k < BS; k++)
+        v[k] = fill ? 0.0 : __ldcg(A + ((size_t)p * BS * BS + r * BS + k) * B + b);
+}
+
+template <int BS, bool SYM>
+__global__ void __launch_bounds__(32 * BS) k_bf_update_rows(const DevSymK S, int B, double *T, double *TU,
+                                                            double *L, const double *U, int *neg,
+                                                            int *bad, double tiny, int t0) {
+    __shared__ double s_d[BS * BS][32];
+    const int lane = threadIdx.x, r = threadIdx.y, b = blockIdx.y * 32 + lane;
+    const bool live = b < B;
+    const int t = t0 + blockIdx.x, p = __ldg(S.tgt_blk + t);
+    const bool diag = p == __ldg(S.tgt_diag + t);
+    const int64_t q0 = __ldg(S.tptr + t), q1 = __ldg(S.tptr + t + 1);
+    if (q0 == q1 && !diag) return;
+    double acc[BS], accU[BS];
+    if (live) {
+        own_row<BS>(S, T, t, p, B, b, r, acc);
+        if (!SYM && !diag) own_row<BS>(S, TU, t, p, B, b, r, accU);
+        row_sums<BS, SYM>(S, B, b, r, q0, q1, T, L, U, !diag, acc, accU);
+#pragma unroll
+        for (int k = 0; k < BS; k++) {
+            if (q0 != q1) T[((size_t)p * BS * BS + r * BS + k) * B + b] = acc[k];
+            if (!SYM && !diag) TU[((size_t)p * BS * BS + r * BS + k) * B + b] = accU[k];
+            if (diag) s_d[r * BS + k][lane] = acc[k];
+        }
+    }
+    if (!diag) return;   // uniform over the block
+    __syncthreads();
+    if (r != 0 || !live) return;
+    double D[BS * BS];
+#pragma unroll
+    for (int e = 0; e < BS * BS; e++) D[e] = s_d[e][lane];
+    finish_pivot<BS>(L, p, B, b, D, neg, bad, tiny);
+}
+
 // ---- split variants: the terms of one target (or one column's sweep) divided among kSlices warps of
 // a block that holds 32 states; slice w takes every kSlices-th term from the w-th, and the slices'
 // partial sums are added in slice order, an entry or two per warp (one warp alone would be at it
@@ -430,6 +509,15 @@ __global__ void __launch_bounds__(kNT) k_bf_backward(const DevSymK S, int B, con
     for (int i = 0; i < BS; i++) x[((size_t)J * BS + i) * B + b] = v[i];
 }
 
+// (i, j), j <= i, of e = i (i + 1) / 2 + j.
+__device__ __forceinline__ void lower_pair(int e, int *pi, int *pj) {
+    int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+    while (i * (i + 1) / 2 > e) i--;
+    while ((i + 1) * (i + 2) / 2 <= e) i++;
+    *pi = i;
+    *pj = e - i * (i + 1) / 2;
+}
+
 // BS values v[0], v[step], .. to consecutive, aligned doubles.
 template <int BS>
 __device__ __forceinline__ void store_col(double *p, const double *v, int step) {
@@ -453,10 +541,8 @@ __global__ void __launch_bounds__(kNT) k_bf_tail(const DevSymK S, int B, const d
     const int b = blockIdx.y * kNT + threadIdx.x;
     if (b >= B) return;
     const int e = blockIdx.x;
-    int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);   // e = i (i + 1) / 2 + j
-    while (i * (i + 1) / 2 > e) i--;
-    while ((i + 1) * (i + 2) / 2 <= e) i++;
-    const int j = e - i * (i + 1) / 2;
+    int i, j;
+    lower_pair(e, &i, &j);
     double acc[BB], accU[BB];
 #pragma unroll
     for (int k = 0; k < BB; k++) { acc[k] = 0.0; accU[k] = 0.0; }
@@ -496,6 +582,39 @@ __global__ void __launch_bounds__(kNT) k_bf_tail(const DevSymK S, int B, const d
     }
 }
 
+// k_bf_tail for small batches (k_bf_update_rows says why).
+template <int BS, bool SYM>
+__global__ void __launch_bounds__(32 * BS) k_bf_tail_rows(const DevSymK S, int B, const double *T,
+                                                          const double *TU, const double *L,
+                                                          const double *U, double *D, double *V,
+                                                          size_t dstride) {
+    const int r = threadIdx.y, b = blockIdx.y * 32 + threadIdx.x;
+    if (b >= B) return;
+    int i, j;
+    lower_pair(blockIdx.x, &i, &j);
+    double acc[BS], accU[BS];
+#pragma unroll
+    for (int k = 0; k < BS; k++) { acc[k] = 0.0; accU[k] = 0.0; }
+    const int t = __ldg(S.tail_tgt + blockIdx.x);
+    if (t >= 0) {
+        const int p = __ldg(S.tgt_blk + t);
+        own_row<BS>(S, T, t, p, B, b, r, acc);
+        if (!SYM) own_row<BS>(S, TU, t, p, B, b, r, accU);
+        row_sums<BS, SYM>(S, B, b, r, __ldg(S.tptr + t), __ldg(S.tail_q1 + t), T, L, U, i != j, acc, accU);
+    }
+    const int n = S.tail_n, r0 = BS * i, c0 = BS * j;
+    double *Db = D + (size_t)b * dstride, *Vb = SYM ? nullptr : V + (size_t)b * dstride;
+#pragma unroll
+    for (int c = 0; c < BS; c++) Db[tail_pos(n, r0 + r, c0 + c)] = acc[c];
+    if (SYM || i == j) return;
+    if ((r0 >> 6) == (c0 >> 6)) {
+#pragma unroll
+        for (int c = 0; c < BS; c++) Db[tail_pos(n, c0 + r, r0 + c)] = accU[c];
+    } else {
+        store_col<BS>(Vb + tail_pos(n, r0, c0 + r), accU, 1);
+    }
+}
+
 // Identity in the rows that pad the tail to a multiple of 64: one thread per entry and state.
 __global__ void __launch_bounds__(kNT) k_bf_tail_pad(int n, int nreal, double *D, double *V,
                                                      size_t dstride) {
@@ -511,29 +630,39 @@ __global__ void __launch_bounds__(kNT) k_bf_tail_pad(int n, int nreal, double *D
     if (V && (row >> 6) == (col >> 6) && col < nreal) D[b * dstride + tail_pos(n, col, row)] = 0.0;
 }
 
-// Right-hand side of the tail: r_J - sum over K < k0 of F_JK z_K, one thread per (state, column).
+// Right-hand side of the tail: r_J - sum over K < k0 of F_JK z_K, one block of kSlices warps per (32
+// states, column), the slices' sums added in slice order.
 template <int BS>
-__global__ void __launch_bounds__(kNT) k_bf_tail_rhs(const DevSymK S, int B, const double *T, double *x) {
-    const int b = blockIdx.y * kNT + threadIdx.x;
-    if (b >= B) return;
+__global__ void __launch_bounds__(32 * kSlices) k_bf_tail_rhs(const DevSymK S, int B, const double *T,
+                                                              double *x) {
+    __shared__ double part[kSlices][BS][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, b = blockIdx.y * 32 + lane;
+    const bool live = b < B;
     const int J = S.k0 + blockIdx.x;
     double y[BS];
 #pragma unroll
-    for (int i = 0; i < BS; i++) y[i] = __ldcg(x + ((size_t)J * BS + i) * B + b);
-    for (int64_t r = __ldg(S.rowptr + J), r1 = __ldg(S.tail_r1 + J); r < r1; r++) {
-        const int K = __ldg(S.rowcol + r), p = __ldg(S.rowblk + r);
-        if (!EXAGO_DCHECK(S, K >= 0 && K < S.nb && p >= 0 && p < S.nblk)) continue;
-        double F[BS * BS], z[BS];
-        load_blk<BS>(T, p, B, b, F);
+    for (int i = 0; i < BS; i++) y[i] = 0.0;
+    if (live)
+        for (int64_t r = __ldg(S.rowptr + J) + w, r1 = __ldg(S.tail_r1 + J); r < r1; r += kSlices) {
+            const int K = __ldg(S.rowcol + r), p = __ldg(S.rowblk + r);
+            if (!EXAGO_DCHECK(S, K >= 0 && K < S.nb && p >= 0 && p < S.nblk)) continue;
+            double F[BS * BS], z[BS];
+            load_blk<BS>(T, p, B, b, F);
 #pragma unroll
-        for (int i = 0; i < BS; i++) z[i] = __ldcg(x + ((size_t)K * BS + i) * B + b);
+            for (int i = 0; i < BS; i++) z[i] = __ldcg(x + ((size_t)K * BS + i) * B + b);
 #pragma unroll
-        for (int i = 0; i < BS; i++)
+            for (int i = 0; i < BS; i++)
 #pragma unroll
-            for (int k = 0; k < BS; k++) y[i] = fma(-F[i * BS + k], z[k], y[i]);
-    }
+                for (int k = 0; k < BS; k++) y[i] = fma(-F[i * BS + k], z[k], y[i]);
+        }
 #pragma unroll
-    for (int i = 0; i < BS; i++) x[((size_t)J * BS + i) * B + b] = y[i];
+    for (int i = 0; i < BS; i++) part[w][i][lane] = y[i];
+    __syncthreads();
+    if (w >= BS || !live) return;
+    double s = part[0][w][lane];
+#pragma unroll
+    for (int v = 1; v < kSlices; v++) s += part[v][w][lane];
+    x[((size_t)J * BS + w) * B + b] = __ldcg(x + ((size_t)J * BS + w) * B + b) + s;
 }
 
 }  // namespace
@@ -541,7 +670,7 @@ __global__ void __launch_bounds__(kNT) k_bf_tail_rhs(const DevSymK S, int B, con
 // A level is split when it has fewer than kSplitBelow targets (factor) or columns (sweeps) and a sum of
 // more than kSplitTerms terms: properties of the structure, not of the batch.  Levels of short sums
 // were split too: 200 buses x 37 states spent 200 us in 12 sweep launches of a few terms each.
-constexpr int kSplitBelow = 64, kSplitTerms = 6;
+constexpr int kSplitBelow = 64, kSplitTerms = 2;
 
 template <int BS, bool SYM>
 int launch_block_factor(const DevSym &S, int B, double *T, double *TU, double *L, double *U,
@@ -555,6 +684,9 @@ int launch_block_factor(const DevSym &S, int B, double *T, double *TU, double *L
         if (nt < kSplitBelow && S.sp_pairs[l] > kSplitTerms)
             k_bf_update_split<BS, SYM><<<dim3((unsigned)nt, gy32), 32 * kSlices, 0, st>>>(
                 S.k, B, T, TU, L, U, neg, bad, tiny, t0);
+        else if (B < kRowsBelow)
+            k_bf_update_rows<BS, SYM><<<dim3((unsigned)nt, gy32), dim3(32, BS), 0, st>>>(
+                S.k, B, T, TU, L, U, neg, bad, tiny, t0);
         else
             k_bf_update<BS, SYM><<<grid, kNT, 0, st>>>(S.k, B, T, TU, L, U, neg, bad, tiny, t0);
         if (nt > S.sp_cols[l])   // blocks below a diagonal
@@ -565,8 +697,13 @@ int launch_block_factor(const DevSym &S, int B, double *T, double *TU, double *L
         const TailShape ts = tail_shape(n, B, SYM);
         double *D = (double *)((char *)tail + ts.dn);
         double *V = SYM ? nullptr : (double *)((char *)tail + ts.dv);
-        k_bf_tail<BS, SYM><<<dim3((unsigned)(R * (R + 1) / 2), gy), kNT, 0, st>>>(
-            S.k, B, T, TU, L, U, D, V, ts.dense_doubles);
+        const unsigned blocks = (unsigned)(R * (R + 1) / 2);
+        if (B < kRowsBelow)
+            k_bf_tail_rows<BS, SYM><<<dim3(blocks, gy32), dim3(32, BS), 0, st>>>(
+                S.k, B, T, TU, L, U, D, V, ts.dense_doubles);
+        else
+            k_bf_tail<BS, SYM><<<dim3(blocks, gy), kNT, 0, st>>>(S.k, B, T, TU, L, U, D, V,
+                                                                 ts.dense_doubles);
         for (int b0 = 0; n > nreal && b0 < B; b0 += 65535)
             k_bf_tail_pad<<<dim3((unsigned)(((n - nreal) * n + kNT - 1) / kNT),
                                  (unsigned)(B - b0 < 65535 ? B - b0 : 65535)), kNT, 0, st>>>(
@@ -594,7 +731,7 @@ int launch_block_solve(const DevSym &S, int B, const double *T, const double *L,
     }
     if (S.k.tail_n > 0) {
         const int R = S.k.nb - S.k.k0;
-        k_bf_tail_rhs<BS><<<dim3((unsigned)R, gy), kNT, 0, st>>>(S.k, B, T, x);
+        k_bf_tail_rhs<BS><<<dim3((unsigned)R, gy32), 32 * kSlices, 0, st>>>(S.k, B, T, x);
         const int e = launch_tail_solve(tail_shape(S.k.tail_n, B, SYM), B, R * BS, SYM, tail,
                                         x + (size_t)S.k.k0 * BS * B, st);
         if (e != 0) return e;
