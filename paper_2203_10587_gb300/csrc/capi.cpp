@@ -336,6 +336,13 @@ int item_rows_max(exago_net *net, int per_item) {
     return mx;
 }
 
+// Whether the user has left the configuration alone, so that the library may choose.
+bool untouched(const exago_config &c) {
+    return c.schedule == EXAGO_SCHED_AUTO && !c.block && !c.occupancy && !c.stage_records && !c.lag &&
+           !c.ring && !c.chunk && !c.use_graph && !c.spin_limit && !c.test_force_timeout &&
+           !c.tile_group && !c.tiling;
+}
+
 // Whether an untouched configuration runs branch-per-warp tiles: on meshed grids, where a
 // per-thread bus tile's warps run to their highest-degree bus and its rows outgrow the staging.
 // Measured on GB300, per thread against per warp (us; the second pair with generator masks):
@@ -353,9 +360,7 @@ int item_rows_max(exago_net *net, int per_item) {
 // so: three branches a bus and 120,000 branch items, or two and a half and a million; fewer than 32
 // states leave lanes idle.
 bool prefer_warp_tiles(const exago_net *net, const exago_config &c, int B) {
-    if (c.schedule != EXAGO_SCHED_AUTO || c.tiling != EXAGO_TILING_DEFAULT || c.block || c.occupancy ||
-        c.stage_records || c.lag || c.ring || c.tile_group)
-        return false;
+    if (!untouched(c)) return false;
     const double nl = net->plan.nl, items = nl * B;
     if (B < 32) return false;
     return (nl >= 3.0 * net->plan.nb && items >= 1.2e5) || (nl >= 2.5 * net->plan.nb && items >= 1e6);
@@ -432,6 +437,17 @@ Resolved resolve(exago_net *net, int B) {
         r.ring = ring;
         return r;
     }
+    if (pers && untouched(net->cfg) && !net->tuned.count(B)) {
+        // One wave of items: warps are few, so a block with all the registers it wants (12 warps an SM)
+        // and its records in one bulk copy is faster (us, default against this: 10,000 buses x 1
+        // state 27.1, 25.1; x 4 41.2, 35.0; 2,000 x 1 24.7, 22.6; x 16 37.3, 33.5; 500 x 64 36.6, 32.9).
+        // A little over a wave it loses (1,000 x 64 44.4, 46.9; 4,000 x 16 45.2, 55.6).
+        const double items = (double)B * ((std::max(net->plan.nl, net->plan.nb) + 63) / 64);
+        if (items <= (double)net->sm_count * occupancy(net, true, 64, 8, 0)) {
+            r.occ_warps = 8;
+            r.stage_recs = 2;
+        }
+    }
     r.stage_cap = stage_cap(net, pers, r.block, r.occ_warps, r.stage_recs);
     r.grid = net->sm_count * occupancy(net, true, r.block, r.occ_warps,
                                        pers ? (size_t)r.stage_cap * sizeof(double) : 0);
@@ -461,11 +477,7 @@ struct StateBlock {
 
 StateBlock state_block(const exago_net *net, int B) {
     StateBlock s;
-    const exago_config &c = net->cfg;
-    if (c.schedule != EXAGO_SCHED_AUTO || c.block || c.occupancy || c.stage_records || c.lag ||
-        c.ring || c.chunk || c.use_graph || c.spin_limit || c.test_force_timeout ||
-        c.tile_group || c.tiling || net->tuned.count(B))
-        return s;
+    if (!untouched(net->cfg) || net->tuned.count(B)) return s;
     const size_t rec = (size_t)NCOMP * net->dev.nslot * sizeof(double);
     if (rec > (size_t)kStateMaxBytes || net->plan.nl > 1280) return s;
     auto smem_of = [&](int nt, int *cap) {
@@ -478,7 +490,9 @@ StateBlock state_block(const exago_net *net, int B) {
     //   256 threads a state   12 + 0.052 a branch for one block an SM; two resident blocks of a
     //                         further wave take 0.72 of one's time each;
     //   64 threads a state    7.5 + 0.14 a branch, the blocks of an SM overlapping (up to 160
-    //                         branches: one pass of 64 threads takes three items each).
+    //                         branches: one pass of 64 threads takes three items each);
+    //   512 threads a state   12.5 (up to 64 branches), 10 + 0.05 a branch (257 to 512), for one
+    //                         block an SM at most; between those 256 threads are faster.
     // For example 118 x 1,024: 77, 100 and 60 (measured 70, 73 and 68); 300 x 304: 64, 46 (68,
     // 47); 900 x 304: 145, 146 (129, 143).
     const double nl = net->plan.nl, per_sm = (double)B / (net->sm_count > 0 ? net->sm_count : 1);
@@ -489,7 +503,13 @@ StateBlock state_block(const exago_net *net, int B) {
     const double pers = 24.0 + 0.34e-3 * nl * B;
     const double t256 = (12.0 + 0.052 * nl) * (waves <= 1.0 ? 1.0 : two ? 0.72 * waves : waves);
     const double t64 = nl > 160 ? 1e30 : (7.5 + 0.14 * nl) * std::max(1.0, 0.6 + 0.22 * per_sm);
-    if (std::min(t64, t256) >= pers) return s;
+    const double t512 = waves > 1.0 ? 1e30 : nl <= 64 ? 12.5 : nl > 256 && nl <= 512 ? 10.0 + 0.05 * nl : 1e30;
+    if (std::min(std::min(t64, t256), t512) >= pers) return s;
+    if (t512 <= std::min(t64, t256)) {
+        s.nt = 512;
+        s.smem = rec;
+        return s;
+    }
     s.nt = t64 < t256 ? 64 : 256;
     s.cap = t64 < t256 ? cap64 : cap256;
     s.smem = t64 < t256 ? b64 : b256;

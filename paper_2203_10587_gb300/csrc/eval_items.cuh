@@ -622,21 +622,20 @@ struct TileRows {
 // record (consecutive slots are consecutive records, so a warp's loads are coalesced), keeps its
 // diagonal components in dg[0 .. kDiagComps) of shared memory, and -- if the slot leads its
 // neighbour group -- sums the group's later parallel branches in slot order and writes the
-// neighbour's row entries, exactly as bus_item does.
-template <int WANT>
-__device__ __forceinline__ void slot_item(const DevNet &N, int s, const double *scr, double *dg,
-                                          const TileRows &T) {
-    constexpr bool WG = WANT & W_G, WJ = WANT & W_J, WH = WANT & W_H;
+// neighbour's row entries, exactly as bus_item does (slot_rows; SMEM: the records are in shared
+// memory; own: slot s's, already read).
+template <int WANT, bool SMEM>
+__device__ __forceinline__ void slot_rows(const DevNet &N, int s, const double *scr, const TileRows &T,
+                                          const Rec *own = nullptr) {
+    constexpr bool WJ = WANT & W_J, WH = WANT & W_H;
     if (!EXAGO_DCHECK(N, s >= 0 && s < N.chk_nslot)) return;
-    Rec o = load_rec<WANT, false>(scr + (size_t)s * NCOMP);
-    if (WG || WJ) { dg[0] = o.pa; dg[1] = o.pu; dg[2] = o.qa; dg[3] = o.qu; }
-    if (WH) { dg[4] = o.haa; dg[5] = o.hua; dg[6] = o.huu; }
     const int pos = __ldg(N.slot_pos + s);
     if (!(WJ || WH) || pos < 0) return;
+    Rec o = own ? *own : load_rec<WANT, SMEM>(scr + (size_t)s * NCOMP);
     const int i = __ldg(N.slot_bus + s), j = __ldg(N.slot_nbr + s);
     const int e = __ldg(N.slot_ptr + i + 1);
     for (int q = s + 1; q < e && __ldg(N.slot_nbr + q) == j; q++)
-        add_group<WANT>(o, load_rec<WANT, false>(scr + (size_t)q * NCOMP));
+        add_group<WANT>(o, load_rec<WANT, SMEM>(scr + (size_t)q * NCOMP));
     const int k = __ldg(N.bus_k + i);
     const BusRows W = T.template of<WANT>(N, i);
     if (WJ) {
@@ -650,6 +649,17 @@ __device__ __forceinline__ void slot_item(const DevNet &N, int s, const double *
             W.HM[k + pos] = o.huv;                            // (Vm_i, Vm_j)
         }
     }
+}
+
+template <int WANT>
+__device__ __forceinline__ void slot_item(const DevNet &N, int s, const double *scr, double *dg,
+                                          const TileRows &T) {
+    constexpr bool WG = WANT & W_G, WJ = WANT & W_J, WH = WANT & W_H;
+    if (!EXAGO_DCHECK(N, s >= 0 && s < N.chk_nslot)) return;
+    const Rec o = load_rec<WANT, false>(scr + (size_t)s * NCOMP);
+    if (WG || WJ) { dg[0] = o.pa; dg[1] = o.pu; dg[2] = o.qa; dg[3] = o.qu; }
+    if (WH) { dg[4] = o.haa; dg[5] = o.hua; dg[6] = o.huu; }
+    slot_rows<WANT, false>(N, s, scr, T, &o);
 }
 
 // Second phase for bus i: the diagonal sums over its slots' components in slot order (the same

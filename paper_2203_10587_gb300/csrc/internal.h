@@ -231,7 +231,7 @@ int persist_w_allow_stage();
 // largest tile's need in doubles, capped at kStageMaxDoubles; a tile above the cap reads its
 // records from global memory and writes its rows directly.
 // Block-per-state schedule (state_block.cu): a state's records and staged rows in one block's
-// shared memory.  nt: 64 or 256 threads; smem: bytes, at most kStateMaxBytes.
+// shared memory.  nt: 64, 256 or 512 threads; smem: bytes, at most kStateMaxBytes.
 constexpr int kStateMaxBytes = 200 << 10;
 int state_allow_smem();
 int launch_eval_state(const DevNet &net, const EvalReq &req, int nt, size_t smem, void *stream);

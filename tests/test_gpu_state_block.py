@@ -40,8 +40,9 @@ def run(ex, net, bt, B, keys):
 
 # branches: below a warp, 64 threads exactly and one more, 256 exactly and one more, several
 # passes, and the limit of 1,280 (more fall back to the persistent schedule)
-@pytest.mark.parametrize("nb,nl,B,shift", [(3, 2, 1, 0.0), (30, 41, 700, 0.0), (48, 64, 5, 0.2),
+@pytest.mark.parametrize("nb,nl,B,shift", [(3, 2, 1, 0.0), (30, 41, 700, 0.0), (30, 41, 5, 0.1), (48, 64, 5, 0.2),
                                            (48, 65, 5, 0.0), (190, 256, 153, 0.0), (190, 257, 90, 0.1),
+                                           (300, 389, 150, 0.1), (400, 512, 140, 0.0), (400, 513, 140, 0.0),
                                            (300, 900, 150, 0.0), (950, 1280, 150, 0.0),
                                            (950, 1281, 150, 0.0)])
 def test_bitwise_equal_to_persistent(ex, nb, nl, B, shift):
