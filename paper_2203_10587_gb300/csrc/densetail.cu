@@ -81,19 +81,24 @@ __device__ __forceinline__ int tile_at(int row, int grp) {
 // Row exponent as stored beside the digits.
 __device__ __forceinline__ int row_exp(int E) { return E >= 2047 ? kFlag : E - 1022; }
 
-// The digit sums of one target put together: sum_g D_g 512^(12 - g) = W 2^68 + less, |W| < 2^63.
-// Rounded: a floor would bias every sum (measured on a power-flow tail: 25 times the error).
-__device__ __forceinline__ long long join_sums(const float *d) {
+// The digit sums of one target put together: sum_g D_g 512^(12 - g) = W 2^(63 + shift) + less, |W| < 2^62.
+// The unit 2^63 is 2^-61 of the rows' bounds; where the sum is too large for it (which digits near
+// their bound in every place would need) it is rounded to 64 units.  A fixed unit of 2^-56 made the
+// 200-bus KKT step, whose rows' entries range over five decades, 1.7 times as far off as in FP64,
+// and a floor in place of the rounding made it 25 times on a power flow.
+__device__ __forceinline__ long long join_sums(const float *d, int *shift) {
     const int i5 = __float2int_rn(fmaf(d[6], 1.0f / 512.0f, d[5]));
     const int i4 = __float2int_rn(d[4]), i3 = __float2int_rn(d[3]), i2 = __float2int_rn(d[2]);
     const int i1 = __float2int_rn(d[1]), i0 = __float2int_rn(d[0]);
     const long long hi = (long long)i0 * (1 << 18) + ((long long)i1 * 512 + i2);
     const long long lo = (long long)i3 * (1 << 18) + ((long long)i4 * 512 + i5);
-    return hi * (1 << 22) + ((lo + 16) >> 5);
+    const bool wide = (unsigned long long)(hi + (1ll << 34)) >> 35;   // |hi| >= 2^34
+    *shift = wide ? 6 : 0;
+    return wide ? hi * (1 << 21) + ((lo + 32) >> 6) : hi * (1 << 27) + lo;
 }
 
-// Exponent field of what one unit of W weighs for rows of exponents ea and eb: 2^(ea + eb - 56).
-__device__ __forceinline__ int unit_field(int ea, int eb) { return ea + eb + (1023 - 56); }
+// Exponent field of what one unit of W weighs for rows of exponents ea and eb: 2^(ea + eb - 61).
+__device__ __forceinline__ int unit_field(int ea, int eb) { return ea + eb + (1023 - 61); }
 
 // W 2^(f - 1023) as a double, rounded to nearest, on the integer pipe: a conversion instruction
 // takes as long on the FP64 pipe as the addition that follows (64 cycles a warp), these twenty
@@ -256,7 +261,9 @@ __device__ __forceinline__ void take_product(uint32_t tmem, int c0, int ea, cons
                 float v[kDigits];
 #pragma unroll
                 for (int g = 0; g < kDigits; g++) v[g] = d[g][c];
-                const double w = weigh(join_sums(v), unit_field(ea, eb[c0 + 8 * q + 4 * h + c]));
+                int shift;
+                const long long W = join_sums(v, &shift);
+                const double w = weigh(W, unit_field(ea, eb[c0 + 8 * q + 4 * h + c]) + shift);
                 acc[4 * h + c] = sub ? acc[4 * h + c] - w : w;
             }
         }
@@ -451,7 +458,8 @@ constexpr int kFacThreads = 256;
 constexpr int kPitch = 65;   // doubles per column in shared memory: rows of a column and columns
                              // of a row both spread over the banks
 
-// Digits of the 64 x 64 matrix X (shared memory, X[k * kPitch + row]) with one exponent per row.
+// Digits of the 64 x 64 unit lower triangular X (shared memory, X[k * kPitch + row] below the diagonal)
+// with one exponent per row.
 __device__ __forceinline__ void panel_digits(const double *X, char *out, int *xout) {
     for (int it = threadIdx.x; it < 512; it += kFacThreads) {
         const int row = it >> 3, grp = it & 7;
@@ -459,7 +467,8 @@ __device__ __forceinline__ void panel_digits(const double *X, char *out, int *xo
         int E = 1;
 #pragma unroll
         for (int k = 0; k < 8; k++) {
-            v[k] = X[(8 * grp + k) * kPitch + row];
+            const int col = 8 * grp + k;
+            v[k] = row > col ? X[col * kPitch + row] : row == col ? 1.0 : 0.0;
             E = max(E, exp_field(v[k]));
         }
         for (int h = 1; h < 8; h <<= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, h));
@@ -471,9 +480,11 @@ __device__ __forceinline__ void panel_digits(const double *X, char *out, int *xo
     }
 }
 
-// X = M^-1 for the unit lower triangular M held in shared memory by columns (M[k * kPitch + i],
-// zero for i <= k); warp w owns columns w, w + 8, ..; lo / hi: rows lane and lane + 32.
+// X = M^-1 for a unit lower triangular M in shared memory: entry (i, k), i > k, at M[k * kPitch + i] or
+// (T) at M[i * kPitch + k].  Warp w owns columns w, w + 8, ..; lo / hi: rows lane and lane + 32.
+template <bool T>
 __device__ __forceinline__ void unit_inverse(const double *M, int warp, int lane, double *lo, double *hi) {
+    auto at = [&](int i, int k) { return i > k ? (T ? M[i * kPitch + k] : M[k * kPitch + i]) : 0.0; };
 #pragma unroll
     for (int c = 0; c < 8; c++) {
         const int j = warp + 8 * c;
@@ -481,7 +492,7 @@ __device__ __forceinline__ void unit_inverse(const double *M, int warp, int lane
         hi[c] = j == lane + 32 ? 1.0 : 0.0;
     }
     for (int k = 0; k < 31; k++) {
-        const double ml = M[k * kPitch + lane], mh = M[k * kPitch + lane + 32];
+        const double ml = at(lane, k), mh = at(lane + 32, k);
 #pragma unroll
         for (int c = 0; c < 4; c++)
             if (warp + 8 * c <= k) {
@@ -491,7 +502,7 @@ __device__ __forceinline__ void unit_inverse(const double *M, int warp, int lane
             }
     }
     for (int k = 31; k < 63; k++) {
-        const double mh = M[k * kPitch + lane + 32];
+        const double mh = at(lane + 32, k);
 #pragma unroll
         for (int c = 0; c < 8; c++)
             if (warp + 8 * c <= k) {
@@ -530,12 +541,12 @@ __device__ __forceinline__ double reciprocal(double d) {
 // Bound by the FP64 pipe (about 5,000 warp instructions of 64 cycles over four pipes) and, for
 // few states, by the chain of pivots: 192 us for 512 states (290 before the look-ahead), 72 for 37.
 template <bool SYM, int BS>
-__global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 3) k_dt_factor(int n, int J, double *D, double *V,
+__global__ void __launch_bounds__(kFacThreads, 4) k_dt_factor(int n, int J, double *D, double *V,
                                                            size_t dstride, double *dinv, char *linv,
                                                            int *line, char *uinv, int *uine,
                                                            int *neg, int *bad, double tiny) {
     extern __shared__ double sm[];
-    double *Ls = sm, *Us = SYM ? nullptr : sm + 64 * kPitch;
+    double *Ls = sm;   // L by columns, Ls[k * kPitch + i], i > k; LU: row k of D U at Ls[j * kPitch + k]
     __shared__ double s_f[2][64], s_d[64], s_r[64];
     __shared__ unsigned long long s_max[64];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -563,8 +574,9 @@ __global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 3) k_dt_factor(int n, i
         const double fl = lane > k ? lo[c] : 0.0, fh = lane + 32 > k ? hi[c] : 0.0;
         s_f[k & 1][lane] = fl;
         s_f[k & 1][lane + 32] = fh;
-        Ls[k * kPitch + lane] = lane > k ? fl * r : 0.0;
-        Ls[k * kPitch + lane + 32] = lane + 32 > k ? fh * r : 0.0;
+        const double ll = fl * r, lh = fh * r;
+        if (lane > k) Ls[k * kPitch + lane] = ll;
+        if (lane + 32 > k) Ls[k * kPitch + lane + 32] = lh;
         if (lane == 0) {
             s_d[k] = d;
             s_r[k] = r;
@@ -580,8 +592,8 @@ __global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 3) k_dt_factor(int n, i
         for (int w = 0; w < 8; w++) {
             const int k = 8 * c + w;
             __syncthreads();
-            const double fl = SYM ? s_f[k & 1][lane] : Ls[k * kPitch + lane];
-            const double fh = SYM ? s_f[k & 1][lane + 32] : Ls[k * kPitch + lane + 32];
+            const double fl = SYM ? s_f[k & 1][lane] : lane > k ? Ls[k * kPitch + lane] : 0.0;
+            const double fh = SYM ? s_f[k & 1][lane + 32] : lane + 32 > k ? Ls[k * kPitch + lane + 32] : 0.0;
             auto update = [&](int q) {   // column warp + 8 q > k loses column k's part
                 const int j = warp + 8 * q;
                 double u;   // SYM: F's column times L's row; else L's column times the row of D U
@@ -589,7 +601,7 @@ __global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 3) k_dt_factor(int n, i
                     u = Ls[k * kPitch + j];
                 } else {
                     u = __shfl_sync(0xffffffffu, c < 4 ? lo[q] : hi[q], k & 31);
-                    if (lane == 0) Us[k * kPitch + j] = u;   // D U, scaled at the end
+                    if (lane == 0) Ls[j * kPitch + k] = u;   // D U, scaled at the end
                 }
                 if (c < 4 && (!SYM || q < 4)) lo[q] = fma(-fl, u, lo[q]);
                 hi[q] = fma(-fh, u, hi[q]);
@@ -610,10 +622,6 @@ __global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 3) k_dt_factor(int n, i
 #pragma unroll
             for (int q = c + 1; q < 8; q++)
                 if (q > c + 1 || w < 7 || warp > 0) update(q);
-            if (!SYM)
-#pragma unroll
-                for (int q = 0; q <= c; q++)
-                    if (lane == 0 && warp + 8 * q <= k) Us[k * kPitch + warp + 8 * q] = 0.0;
         }
     }
     __syncthreads();
@@ -629,24 +637,29 @@ __global__ void __launch_bounds__(kFacThreads, SYM ? 4 : 3) k_dt_factor(int n, i
         if (lane == 0 && nb) atomicAdd(bad + st, nb);
     }
     if (!SYM) {
-        for (int e = tid; e < 64 * 64; e += kFacThreads) Us[(e >> 6) * kPitch + (e & 63)] *= s_r[e >> 6];
+        for (int e = tid; e < 64 * 64; e += kFacThreads)
+            if ((e >> 6) > (e & 63)) Ls[(e >> 6) * kPitch + (e & 63)] *= s_r[e & 63];
         __syncthreads();
     }
-    for (int side = 0; side < (SYM ? 1 : 2); side++) {
-        double *M = side ? Us : Ls;
-        double *out = side ? V + st * dstride + tail_pos(n, 64 * J, 64 * J) : Dp;
-        unit_inverse(M, warp, lane, lo, hi);
+    // the inverses of L and (LU) of U'; each takes L's place in shared memory
+    auto finish = [&](double *out, char *digits, int *exps) {
         __syncthreads();
 #pragma unroll
         for (int c = 0; c < 8; c++) {
             const int j = warp + 8 * c;
-            M[j * kPitch + lane] = lo[c];
-            M[j * kPitch + lane + 32] = hi[c];
+            if (lane > j) Ls[j * kPitch + lane] = lo[c];
+            if (lane + 32 > j) Ls[j * kPitch + lane + 32] = hi[c];
             out[(size_t)j * ld + lane] = lo[c];
             out[(size_t)j * ld + lane + 32] = hi[c];
         }
         __syncthreads();
-        panel_digits(M, (side ? uinv : linv) + st * kDigits * kTile, (side ? uine : line) + st * 64);
+        panel_digits(Ls, digits + st * kDigits * kTile, exps + st * 64);
+    };
+    unit_inverse<false>(Ls, warp, lane, lo, hi);
+    finish(Dp, linv, line);
+    if (!SYM) {
+        unit_inverse<true>(Ls, warp, lane, lo, hi);
+        finish(V + st * dstride + tail_pos(n, 64 * J, 64 * J), uinv, uine);
     }
 }
 
@@ -697,11 +710,16 @@ __global__ void __launch_bounds__(kSolThreads) k_dt_solve(int n, int nreal, int 
             sx[j0 + tid] = ((part[tid] + part[64 + tid]) + (part[128 + tid] + part[192 + tid])) *
                            __ldg(di + j0 + tid);
         __syncthreads();
+        // four sums of 16 terms, then one subtraction: shorter chains, and fewer roundings at the
+        // size of the target
         for (int i = 64 + tid; i < ld; i += kSolThreads) {
-            double v = sx[j0 + i];
-#pragma unroll 8
-            for (int k = 0; k < 64; k++) v = fma(-__ldg(Dp + (size_t)k * ld + i), sx[j0 + k], v);
-            sx[j0 + i] = v;
+            double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+            for (int k = 0; k < 64; k += 4)
+#pragma unroll
+                for (int h = 0; h < 4; h++)
+                    a[h] = fma(__ldg(Dp + (size_t)(k + h) * ld + i), sx[j0 + k + h], a[h]);
+            sx[j0 + i] -= (a[0] + a[1]) + (a[2] + a[3]);
         }
         __syncthreads();
     }
@@ -741,7 +759,7 @@ __global__ void __launch_bounds__(kSolThreads) k_dt_solve(int n, int nreal, int 
 
 size_t round256(size_t v) { return (v + 255) / 256 * 256; }
 
-size_t fac_smem(bool sym) { return (sym ? 1 : 2) * 64 * kPitch * sizeof(double); }
+size_t fac_smem() { return 64 * kPitch * sizeof(double); }
 
 }  // namespace
 
@@ -783,7 +801,6 @@ int tail_allow_smem() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dt_update<false, 0>, a, kSmemUpd);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dt_update<false, 1>, a, kSmemUpd);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dt_update<false, 2>, a, kSmemUpd);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dt_factor<false, 2>, a, (int)fac_smem(false));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dt_solve<true>, a, 200 << 10);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dt_solve<false>, a, 200 << 10);
     return (int)e;
@@ -807,10 +824,10 @@ int launch_tail_factor(const TailShape &S, int B, int BS, bool sym, void *w, int
                          sym ? linv : uinv, sym ? line : uine, S.digit_bytes, status};
             if (J > 0) k_dt_update<true, 0><<<dim3(1, nB), kUpdThreads, kSmemUpd, st>>>(a);
             if (sym)
-                k_dt_factor<true, 4><<<nB, kFacThreads, fac_smem(true), st>>>(
+                k_dt_factor<true, 4><<<nB, kFacThreads, fac_smem(), st>>>(
                     n, J, D, V, S.dense_doubles, dinv, linv, line, uinv, uine, neg + b0, bad + b0, tiny);
             else
-                k_dt_factor<false, 2><<<nB, kFacThreads, fac_smem(false), st>>>(
+                k_dt_factor<false, 2><<<nB, kFacThreads, fac_smem(), st>>>(
                     n, J, D, V, S.dense_doubles, dinv, linv, line, uinv, uine, neg + b0, bad + b0, tiny);
             const dim3 grid((P - J) / 2, nB);   // 128-row tiles of the P - 1 - J below
             if (grid.x == 0) continue;

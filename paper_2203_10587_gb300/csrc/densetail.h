@@ -15,8 +15,8 @@
 //     tcgen05.mma into 7 FP32 accumulators in TMEM, one per s + t.  The sums with s + t <= 3 stay
 //     within 2^24, so they are exact; the later ones would need digits near their bound in every
 //     place to round at all, and their weight is 2^-36 and less.  The dropped pairs weigh 2^-63.
-//   * The seven sums are put together in 64-bit integers (unit 2^-56 of the rows' bounds) and one
-//     FP64 fused multiply-add takes the 64 products' sum from the target, where the FP64 path
+//   * The seven sums are put together in 64-bit integers (unit 2^-61 of the rows' bounds) and one
+//     FP64 subtraction takes the 64 products' sum from the target, where the FP64 path
 //     rounds 64 times.
 //
 // GB300's FP64 pipe retires 528 G multiply-adds/s (measured), so the 76 M of one state's tail
