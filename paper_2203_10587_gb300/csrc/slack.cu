@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <new>
 #include <string>
 #include <vector>
@@ -292,12 +293,25 @@ exago_status exago_eval_slack(exago_slack_t s, const exago_batch *bt, const doub
                 s->nz, 0, 0, gh ? (nused + kLanes - 1) / kLanes : 0,
                 grad_z ? (s->nz + kPart - 1) / kPart : 0,
                 s->d_cost, z, bt->obj_weight, gh, f, grad_z, ldgh};
-    for (int b0 = 0; b0 < bt->B && (gh || f || grad_z); b0 += kMaxGridY) {
-        A.b0 = b0;
-        A.nB = std::min(kMaxGridY, bt->B - b0);
-        k_slack_apply<<<dim3(kStates + A.row_blocks + A.grad_blocks, (A.nB + kStates - 1) / kStates),
-                        kLanes, 0, stream>>>(A);
-    }
+    auto launch = [&](const SlackArgs &L) {
+        for (int b0 = 0; b0 < bt->B && (L.gh || L.f || L.grad_z); b0 += kMaxGridY) {
+            SlackArgs C = L;
+            C.b0 = b0;
+            C.nB = std::min(kMaxGridY, bt->B - b0);
+            k_slack_apply<<<dim3(kStates + C.row_blocks + C.grad_blocks, (C.nB + kStates - 1) / kStates),
+                            kLanes, 0, stream>>>(C);
+        }
+    };
+    const uintptr_t span = (uintptr_t)bt->B * s->nz * sizeof(double), dist = (uintptr_t)grad_z - (uintptr_t)z;
+    if (grad_z && (gh || f) && (dist < span || -dist < span)) {   // the gradient replaces z: last
+        SlackArgs G = A;
+        G.gh = G.f = nullptr;
+        G.row_blocks = 0;
+        A.grad_z = nullptr;
+        A.grad_blocks = 0;
+        launch(A);
+        launch(G);
+    } else launch(A);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return set_last_error(EXAGO_ECUDA, std::string("slack launch: ") + cudaGetErrorString(e));
