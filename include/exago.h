@@ -601,7 +601,8 @@ exago_status exago_serve_drive(exago_server_t server, const exago_serve_client *
  * them (hval [B][nnzH], the lower triangle; jval [B][nnzJ]).  The flow rows and the generator
  * variables are eliminated first (they create no fill), then the remaining 4 x 4 block per bus
  * (Va, Vm, lamP, lamQ) is factored by a batched block L D L' without pivoting on a minimum-degree
- * order of the bus graph computed once by exago_kkt_create.  K must be factorable without
+ * order of the bus graph computed once by exago_kkt_create (the last columns, where the factor is
+ * nearly full, as one dense matrix per state, with the same pivots in the same order).  K must be factorable without
  * pivoting: it is whenever W + diag(dx) is positive definite and dc > 0 (a quasi-definite K;
  * interior-point methods regularise to that), and dx of every Qg must be nonzero.
  *   exago_kkt_create      symbolic analysis on the host (ordering, factor structure, update
@@ -613,8 +614,9 @@ exago_status exago_serve_drive(exago_server_t server, const exago_serve_client *
  *                         level (0 at the leaves; columns of one level are factored together).
  *   exago_kkt_info        factor blocks, update pairs (4 x 4 block products per state), levels of
  *                         the elimination tree, and FP64 flops of one state's factor and solve.
- *   exago_kkt_workspace_size  scratch bytes for B states (two factor arrays of 16 blocks x 8 B x B
- *                         per factor block, the reduced vectors and counters).
+ *   exago_kkt_workspace_size  scratch bytes for B states (two factor arrays of 16 x 8 B x B per
+ *                         factor block, one without the dense last columns, whose panels and
+ *                         split operands come beside them; the reduced vectors and counters).
  *   exago_kkt_solve       DEVICE pointers, row-major per state: jval [B][nnzJ], hval [B][nnzH],
  *                         dx [B][n], dc [B][m] (> 0), rhs [B][n + m]; sol [B][n + m] receives
  *                         [dx; dlam].  inertia [B][2] (or NULL) receives the number of negative
@@ -648,7 +650,8 @@ exago_status exago_kkt_solve(exago_kkt_t kkt, int B, const double *jval, const d
  *   exago_pf_create          validates bus_type (host [nb], values 1..3, at least one slack) and
  *                            runs the symbolic analysis; the net must have a device and outlive
  *                            the handle.
- *   exago_pf_workspace_size  scratch bytes for B states (g, J, four factor arrays, vectors).
+ *   exago_pf_workspace_size  scratch bytes for B states (g, J, the factor arrays and dense last
+ *                            columns as in exago_kkt_workspace_size, lower and upper, vectors).
  *   exago_pf_step            x_new [B][n] (DEVICE; may equal batch->x) = x + d, Pg and Qg copied;
  *                            mismatch [B] (or NULL) = max |g_pf(x)| before the step.
  *                            batch->workspace: at least exago_pf_workspace_size bytes, or NULL for

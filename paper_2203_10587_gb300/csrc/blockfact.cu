@@ -1,15 +1,16 @@
-// Batched numeric block factorisation and solve (blockfact.h), one thread per (state, target
-// block) per level of the elimination tree.
+// Batched numeric block factorisation and solve (blockfact.h).  The columns below k0 go level by
+// level of the elimination tree, one thread per (state, target block) or a few (below); the last
+// ones, the dense tail, get their updates by those columns here and are then factored as one
+// matrix per state (densetail.h), which holds most of the work of a large grid.
 //
 // Factor, per level: every target (I, J) of the level's columns accumulates its left-looking
 // update T_IJ = A_IJ - sum_K F_IK U_KJ (SYM: U_KJ = L_JK') in registers, in the pair order the
-// host fixed (ascending K), and stores it; then every target rescales by the inverse of its
-// column's pivot block D_J = T_JJ (L_IJ = T_IJ D_J^-1; LU: U_JI = D_J^-1 T'_JI; the diagonal
-// position of L receives D_J^-1).  The pivot block is inverted by Gauss-Jordan elimination
-// without pivoting, in the same order by every thread of its column, so all of them use bitwise
-// the same inverse.  Solve: forward y_J = r_J - sum_K F_JK z_K, z_J = D_J^-1 y_J over ascending
-// levels (F = L D is what the factor kept in T), then backward x_J = z_J - sum_I U_JI x_I over
-// descending levels.
+// host fixed (ascending K), and stores it (a fill block starts from zero, unread);
+// the diagonal target also inverts its column's pivot block D_J = T_JJ, by Gauss-Jordan
+// elimination without pivoting, into the diagonal position of L; then every other target is
+// scaled by that inverse (L_IJ = T_IJ D_J^-1; LU: U_JI = D_J^-1 T'_JI).  Solve: forward y_J = r_J
+// - sum_K F_JK z_K, z_J = D_J^-1 y_J over ascending levels (F = L D is what the factor kept in T),
+// then backward x_J = z_J - sum_I U_JI x_I over descending levels, the tail's sweeps between.
 // A warp holds 32 consecutive states of one target, so every value load is one coalesced
 // 256-byte access and every index load is uniform across the warp.
 #include <cuda_runtime.h>

@@ -16,7 +16,9 @@
 // The device factors A = L D L' (SYM, symmetric: the KKT step) or A = L D U (the power flow),
 // with unit block-triangular L, U and block-diagonal D, level by level:
 //   T_IJ = A_IJ - sum_K F_IK U_KJ  with F_IK = L_IK D_K  (= the stored T_IK), U_KJ = L_JK' (SYM);
-//   D_J = T_JJ;  L_IJ = T_IJ D_J^-1;  U_JI = D_J^-1 T'_JI (upper targets, LU only).
+//   D_J = T_JJ;  L_IJ = T_IJ D_J^-1;  U_JI = D_J^-1 T'_JI (upper targets, LU only),
+// up to column k0; the columns from there on, where choose_tail finds it cheaper, are one dense
+// matrix per state, factored in 64-column panels (densetail.h).
 // Every value array is batch-interleaved: entry e of block p of state b is at [(p BS^2 + e) B + b],
 // so the threads of a warp (consecutive states) read consecutive doubles.  No atomics on values.
 #pragma once

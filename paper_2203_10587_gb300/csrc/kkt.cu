@@ -12,7 +12,8 @@
 //   2. each generator's Pg (pivot W_kk + dx_k) and Qg (pivot dx) couples only its bus's P or Q
 //      row: eliminating it subtracts a^2 / pivot from that row's diagonal;
 //   3. what remains is one 4 x 4 block per bus, unknowns (Va, Vm, lamP, lamQ), on the bus graph:
-//      factored by the batched block L D L' (blockfact.cu) on a minimum-degree order;
+//      factored by the batched block L D L' (blockfact.cu) on a minimum-degree order, its last
+//      columns as one dense matrix per state (densetail.cu);
 //   4. the eliminated unknowns are recovered from the reduced solution.
 // Per state the factor's negative pivots (1. to 3.) are counted: the inertia an interior-point
 // method checks (m negative pivots for a correct step).

@@ -8,8 +8,8 @@
 // graph: a fixed unknown (Va and Vm of the slack bus, Vm of a PV bus) gets an identity row in
 // place of its bus's inactive balance (P <-> Va, Q <-> Vm) and a zero column, so its step is
 // exactly 0 and the other unknowns solve the reduced system.  The block matrix is not symmetric:
-// it is factored A = L D U without pivoting (blockfact.cu) on the same minimum-degree order of
-// the bus graph as the KKT step.
+// it is factored A = L D U without pivoting (blockfact.cu, densetail.cu) on the same
+// minimum-degree order of the bus graph as the KKT step.
 #include <cuda_runtime.h>
 
 #include <algorithm>
