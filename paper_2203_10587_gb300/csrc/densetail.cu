@@ -18,6 +18,7 @@ constexpr int kEpi = 128 * (64 / kCols);   // such threads
 constexpr int kUpdThreads = kEpi + 32;
 constexpr int kSmemA = kDigits * 2 * kTile, kSmemB = kDigits * kTile;
 constexpr int kSmemUpd = kSmemA + kSmemB + 1024;   // + alignment of the tiles to 1 KB
+constexpr int kHalfSums = kDigits * 32;   // TMEM columns of the 7 sums of 32 columns
 constexpr int kSpin = 1 << 20;        // polls of an mbarrier before a wait gives up
 enum : int { ST_TIMEOUT_TAIL = 4 };
 
@@ -177,22 +178,17 @@ __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, bool add
         : "memory");
 }
 
-// Digit S of the rows times digits 0 .. 6 - S of the columns: their tiles lie one after another
-// in shared memory and the sums S .. 6 in TMEM, so they are one operand of 64 (7 - S) columns (at
-// most 256 an instruction).  40 instructions a step in place of 112 of 64 columns, which one
-// thread could not issue as fast as they ran.
+// Digit S of the rows times digits 0 .. 6 - S of 32 columns: these lie one after another in shared
+// memory and the sums S .. 6 in TMEM, so they are one operand of 32 (7 - S) columns.  28
+// instructions in place of 112 of 32 columns, which one thread could not issue as fast as they ran.
 template <int S>
 __device__ __forceinline__ void issue_digit(uint32_t tmem, uint64_t a, uint64_t b) {
-    constexpr int N = 64 * (kDigits - S), N0 = N > 256 ? 256 : N, N1 = N - N0;
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-        mma<N0>(tmem + 64 * S, a + ((S * 2 * kTile + 32 * k) >> 4), b + ((32 * k) >> 4), S > 0 || k > 0);
-        if (N1 > 0)
-            mma<N1 ? N1 : 64>(tmem + 64 * S + N0, a + ((S * 2 * kTile + 32 * k) >> 4),
-                              b + ((4 * kTile + 32 * k) >> 4), S > 0 || k > 0);
-    }
+    for (int k = 0; k < 4; k++)
+        mma<32 * (kDigits - S)>(tmem + 32 * S, a + ((S * 2 * kTile + 32 * k) >> 4), b + ((32 * k) >> 4),
+                                S > 0 || k > 0);
 }
-// All 28 digit pairs of one 64-deep product, into the 7 sums (64 columns each).
+// All 28 digit pairs of one 64-deep product with 32 columns, into their 7 sums.
 __device__ __forceinline__ void issue_products(uint32_t tmem, uint32_t a0, uint32_t b0) {
     const uint64_t a = mma_desc(a0), b = mma_desc(b0);
     issue_digit<0>(tmem, a, b);
@@ -216,7 +212,7 @@ __device__ __forceinline__ void tmem_sums4(uint32_t addr, float (*v)[4]) {
     for (int g = 0; g < kDigits; g++)
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                      : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3])
-                     : "r"(addr + 64 * g)
+                     : "r"(addr + 32 * g)
                      : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(r[0][0]), "+r"(r[0][1]), "+r"(r[0][2]), "+r"(r[0][3]), "+r"(r[1][0]),
@@ -232,6 +228,10 @@ __device__ __forceinline__ void tmem_sums4(uint32_t addr, float (*v)[4]) {
         for (int c = 0; c < 4; c++) v[g][c] = __uint_as_float(r[g][c]);
 }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpi) : "memory"); }
+// The threads of one half of the columns.
+__device__ __forceinline__ void half_sync(int half) {
+    asm volatile("bar.sync %0, %1;" ::"r"(2 + half), "n"(kEpi / 2) : "memory");
+}
 
 // The thread's values, eight places on: the loops below take eight values at a time from the front,
 // so that their bodies are in the instruction cache once (unrolled over all columns, half of the
@@ -246,12 +246,13 @@ __device__ __forceinline__ void rotate8(double *v) {
     for (int i = 0; i < 8; i++) v[kCols - 8 + i] = t[i];
 }
 
-// acc[0 .. kCols) -= (sub) or = the product in TMEM, this thread's row and kCols columns from c0; ea:
-// the row's exponent, eb [64] the columns' (shared memory).
+// acc[0 .. NC) -= (sub) or = the product in TMEM, this thread's row and NC columns from column c0 of
+// the half; ea: the row's exponent, eb [32] the columns' (shared memory).
+template <int NC>
 __device__ __forceinline__ void take_product(uint32_t tmem, int c0, int ea, const int *eb, double *acc,
                                              bool sub) {
 #pragma unroll 1
-    for (int q = 0; q < kCols / 8; q++) {
+    for (int q = 0; q < NC / 8; q++) {
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             float d[kDigits][4];
@@ -267,7 +268,7 @@ __device__ __forceinline__ void take_product(uint32_t tmem, int c0, int ea, cons
                 acc[4 * h + c] = sub ? acc[4 * h + c] - w : w;
             }
         }
-        rotate8(acc);
+        if (NC > 8) rotate8(acc);
     }
 }
 
@@ -294,15 +295,19 @@ __device__ __forceinline__ size_t digit_at(int P, int K, int s, int I) {
 
 // One tile of 128 rows (DIAG: the panel's own 64) of panel J, one block per (tile, state).
 // MODE 0: F and L (SYM); 1: F alone (LU, lower side); 2: U' from G = U' D' (LU, upper side).
-// What bounds it: the 28 x 4 tensor instructions of a 64-deep step (128 x 64 x 16 each) and, as
-// much, the 8,192 targets' integer joins and two FP64-pipe instructions each; one block per SM
-// (172 KB of digits), 16 warps that finish products beside one that issues copies and MMAs.
+// What bounds it: the 8,192 targets' integer joins and two FP64-pipe instructions each, beside 2.4
+// us of tensor work a 64-deep step; one block per SM (172 KB of digits), 16 warps that finish
+// products beside one that issues copies and MMAs.  The columns go in two halves of 32, each with
+// its sums in TMEM and 8 warps of its own, so that one half's products run while the other's sums
+// are joined: a 64-deep step 6.5 to 8 us (8 with all 64 columns at once), half of it the
+// 172 KB from HBM.  DIAG puts the 64 rows into both halves of the lanes, so that every warp has
+// half the columns: 8.1 to 5.9 us a step.  2,000 buses x 512 states, all launches: 9.8 to 8.7 ms.
 // A wait that gives up sets the status word and the block's flag; the block then runs to its end
 // on whatever it holds, so that every barrier is met.
 template <bool DIAG, int MODE>
 __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A) {
     extern __shared__ char raw[];
-    __shared__ uint64_t bar_full, bar_mma, bar_epi, bar_tgt;
+    __shared__ uint64_t bar_full, bar_mma[2], bar_epi[2], bar_tgt;
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_dead;
     __shared__ int s_eb[2][64], s_em[64 / kCols][128];
@@ -314,8 +319,10 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
     const int tiles = DIAG ? 1 : min(2, P - I0);
     if (tid == 0) {
         mbar_init(&bar_full, 1);
-        mbar_init(&bar_mma, 1);
-        mbar_init(&bar_epi, kEpi);
+        for (int h = 0; h < 2; h++) {
+            mbar_init(&bar_mma[h], 1);
+            mbar_init(&bar_epi[h], kEpi / 2);
+        }
         mbar_init(&bar_tgt, kEpi);
         s_dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -340,19 +347,22 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
             bool ok = true;
             for (int K = 0; K < steps && ok; K++) {
                 const bool last = K == J;
-                if (K > 0) ok = mbar_wait(&bar_mma, (K - 1) & 1, A.status, &s_dead);
+                // both halves' products of the step before: its operands are no longer read
+                if (K > 0) ok = mbar_wait(&bar_mma[1], (K - 1) & 1, A.status, &s_dead);
                 if (!ok) break;   // nothing in flight
-                mbar_expect(&bar_full, last ? kDigits * kTile : kDigits * kTile * (tiles + 1));
+                mbar_expect(&bar_full, last ? kDigits * kTile : kDigits * kTile * (DIAG ? 3 : tiles + 1));
                 for (int s = 0; s < kDigits; s++) {
+                    const char *b = last ? A.inv + (st * kDigits + s) * kTile : sb + digit_at(P, K, s, J);
                     if (!last) {
-                        copy_in(sA + s * 2 * kTile, sa + digit_at(P, K, s, I0), kTile * tiles, &bar_full);
-                        copy_in(sB + s * kTile, sb + digit_at(P, K, s, J), kTile, &bar_full);
-                    } else {
-                        copy_in(sB + s * kTile, A.inv + (st * kDigits + s) * kTile, kTile, &bar_full);
+                        const char *a = sa + digit_at(P, K, s, I0);
+                        copy_in(sA + s * 2 * kTile, a, kTile * tiles, &bar_full);
+                        if (DIAG) copy_in(sA + s * 2 * kTile + kTile, a, kTile, &bar_full);
                     }
+                    for (int h = 0; h < 2; h++)
+                        copy_in(sB + (h * kDigits + s) * (kTile / 2), b + h * (kTile / 2), kTile / 2, &bar_full);
                 }
-                // the product before has left TMEM; the targets' digits are in shared memory
-                if (K > 0) ok = mbar_wait(&bar_epi, (K - 1) & 1, A.status, &s_dead);
+                // the half's product before has left TMEM; the targets' digits are in shared memory
+                if (K > 0) ok = mbar_wait(&bar_epi[0], (K - 1) & 1, A.status, &s_dead);
                 if (last) ok = mbar_wait(&bar_tgt, 0, A.status, &s_dead) && ok;
                 // this wait also holds a block that gave up until its copies have landed
                 volatile int no = 0;
@@ -360,36 +370,45 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
                 if (!ok) { s_dead = 1; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 issue_products(tmem, a0, b0);
-                commit(&bar_mma);
+                commit(&bar_mma[0]);
+                if (K > 0) ok = mbar_wait(&bar_epi[1], (K - 1) & 1, A.status, &s_dead);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                issue_products(tmem + kHalfSums, a0, b0 + kDigits * (kTile / 2));
+                commit(&bar_mma[1]);
             }
         }
         __syncwarp();
     } else {
-        const int part = warp >> 2;                       // columns kCols part ..
-        const int row = ((warp & 3) << 5) | lane, c0 = kCols * part;
+        const int part = warp >> 2, half = part >> 1;     // columns kCols part ..
+        // DIAG: lanes 64 .. 127 hold the 64 rows again and take the last 8 of the 16 columns
+        const int lane128 = ((warp & 3) << 5) | lane, row = DIAG ? lane128 & 63 : lane128;
+        const int c0 = kCols * part + (DIAG ? 8 * (lane128 >> 6) : 0);
         const int grow = 64 * I0 + row;                   // row of the matrix
         const bool live = row < 64 * tiles;
-        const uint32_t tw = tmem + ((uint32_t)(warp & 3) << 21);
+        const uint32_t tw = tmem + ((uint32_t)(warp & 3) << 21) + kHalfSums * half;
         const int ld = n - 64 * J;
         double *Dp = A.D + st * A.dstride + tail_pos(n, 64 * J, 64 * J) + (size_t)c0 * ld +
                      (grow - 64 * J);
-        double acc[kCols];
+        constexpr int NC = DIAG ? 8 : kCols;
+        double acc[kCols] = {};
 #pragma unroll
-        for (int c = 0; c < kCols; c++) acc[c] = live ? __ldcg(Dp + (size_t)c * ld) : 0.0;
+        for (int c = 0; c < NC; c++) acc[c] = live ? __ldcg(Dp + (size_t)c * ld) : 0.0;
         const int *xa = A.xa + st * (size_t)P * n, *xb = A.xb + st * (size_t)P * n;
         const double *dinv = A.dinv + st * n + 64 * J + c0;
         // steps K < J: the products of the panels before; J: the targets times the inverse, F_IJ
         // (MODE 2: U'); J + 1: its digits kept for the panels to come; J + 2: L_IJ's (MODE 0)
         const int steps = DIAG ? J : J + (MODE == 0 ? 3 : 2);
+        const bool mine = (tid & (kEpi / 2 - 1)) < 32;    // one warp of a half keeps its columns' exponents
+        const int col = 32 * half + lane;
 #pragma unroll 1
         for (int K = 0; K < steps; K++) {
             int ea = 0;
             if (DIAG || K < J) {
-                if (tid < 64) s_eb[K & 1][tid] = __ldcg(xb + (size_t)K * n + 64 * J + tid);
+                if (mine) s_eb[K & 1][col] = __ldcg(xb + (size_t)K * n + 64 * J + col);
                 if (live) ea = __ldcg(xa + (size_t)K * n + grow);
-                epi_sync();
+                half_sync(half);
             } else {
-                if (K == J && tid < 64) s_eb[J & 1][tid] = __ldcg(A.inve + st * 64 + tid);
+                if (K == J && mine) s_eb[J & 1][col] = __ldcg(A.inve + st * 64 + col);
                 int E = 1;
 #pragma unroll
                 for (int c = 0; c < kCols; c++) E = max(E, exp_field(acc[c]));
@@ -411,12 +430,12 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
                 if (K == J) mbar_arrive(&bar_tgt);
             }
             if (DIAG || K <= J) {
-                mbar_wait(&bar_mma, K & 1, A.status, &s_dead);
+                mbar_wait(&bar_mma[half], K & 1, A.status, &s_dead);
                 __syncwarp();
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (!DIAG || (warp & 3) < 2) take_product(tw, c0, ea, s_eb[K & 1], acc, K < J);
+                take_product<NC>(tw, c0 & 31, ea, s_eb[K & 1] + 32 * half, acc, K < J);
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                if (DIAG || K < J) mbar_arrive(&bar_epi);
+                if (DIAG || K < J) mbar_arrive(&bar_epi[half]);
                 if (!DIAG && K == J) {
                     if (MODE == 2)
 #pragma unroll
@@ -443,9 +462,9 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
                 epi_sync();
             }
         }
-        if (DIAG && live)
+        if (DIAG)
 #pragma unroll
-            for (int c = 0; c < kCols; c++) Dp[(size_t)c * ld] = acc[c];
+            for (int c = 0; c < NC; c++) Dp[(size_t)c * ld] = acc[c];
     }
     __syncthreads();
     if (warp == kEpi / 32)
