@@ -4,6 +4,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <climits>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -177,6 +178,7 @@ exago_status do_upload(exago_net *net) {
     for (int t = 0; t < 4; t++) {   // largest bus tile's rows (and components), 32 to 256 buses
         const int T = 32 << t;
         int64_t rows = 0, all = 0, bulk = 0;
+        std::vector<int64_t> each;
         for (int i0 = 0; i0 < p.nb; i0 += T) {
             const int i1 = i0 + T < p.nb ? i0 + T : p.nb;
             const int64_t r = 2 * (p.Jrowptr[i1] - p.Jrowptr[i0]) + (p.Hrowptr[i1] - p.Hrowptr[i0]) +
@@ -184,10 +186,17 @@ exago_status do_upload(exago_net *net) {
             const int64_t a = r + (int64_t)kDiagComps * (p.slot_ptr[i1] - p.slot_ptr[i0]);
             const int64_t k = r + (int64_t)NCOMP * (p.slot_ptr[i1] - p.slot_ptr[i0]);
             if (r > rows) rows = r;
+            each.push_back(r);
             if (a > all) all = a;
             if (k > bulk) bulk = k;
         }
         d.stage_cap_rows[t] = (int)(rows < kStageMaxDoubles ? rows : kStageMaxDoubles);
+        d.stage_cap_most[t] = 0;
+        if (!each.empty()) {
+            auto q = each.end() - 1 - each.size() / 16;
+            std::nth_element(each.begin(), q, each.end());
+            d.stage_cap_most[t] = (int)std::min<int64_t>(*q, kStageMaxDoubles);
+        }
         d.stage_cap_all[t] = (int)(all < kStageMaxDoubles ? all : kStageMaxDoubles);
         d.stage_cap_bulk[t] = (int)(bulk < kStageMaxDoubles ? bulk : kStageMaxDoubles);
     }
@@ -304,15 +313,16 @@ int occupancy(exago_net *net, bool persistent, int block, int occ_warps, size_t 
 
 // Shared-memory doubles of one bus tile: its row segments (and, slot-parallel, its slots'
 // diagonal components), but no more than keeps the register-limited number of resident CTAs per
-// SM.  A tile that does not fit writes its rows straight to global memory (and walks its slots
-// per bus).
+// SM, nor more than leaves L1 its share (stage_budget).  A tile that does not fit writes its rows
+// straight to global memory (and walks its slots per bus).
 int stage_cap(exago_net *net, bool persistent, int block, int occ_warps, int stage_recs) {
     const int t = stage_index(persistent ? block : 128);
     const int by_regs = occupancy(net, persistent, block, occ_warps, 0);
-    const long budget = ((long)net->smem_per_sm / (by_regs > 0 ? by_regs : 1) - 4096) / 8;
     const int want = stage_recs == 2   ? net->dev.stage_cap_bulk[t]
                      : stage_recs == 1 ? net->dev.stage_cap_all[t]
                                        : net->dev.stage_cap_rows[t];
+    const long budget = stage_budget(net->smem_per_sm, by_regs, persistent && occ_warps == 8,
+                                     stage_recs == 0 ? net->dev.stage_cap_most[t] : INT_MAX);
     return want > budget ? (int)(budget & ~1l) : want;
 }
 

@@ -773,6 +773,7 @@ void launch_cart_persist(bool ps, int grid, size_t smem, cudaStream_t st, const 
 CartShape cart_shape(const DevNet &N, int occ) {
     const bool ps = N.Gtf != nullptr;
     const int want = std::max(0, N.stage_cap_rows[stage_index(128)]);
+    const int most = N.stage_cap_most[stage_index(128)];
     CartShape sh{0, 152};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
@@ -780,9 +781,9 @@ CartShape cart_shape(const DevNet &N, int occ) {
         return sh;
     }
     static std::mutex mu;
-    static std::map<uint64_t, CartShape> cache;
+    static std::map<uint64_t, CartShape> cache;   // want and most: 14 bits each
     const uint64_t key = ((uint64_t)dev << 48) | ((uint64_t)occ << 40) | ((uint64_t)ps << 32) |
-                         (uint64_t)(uint32_t)want;
+                         ((uint64_t)most << 16) | (uint64_t)want;
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
@@ -795,7 +796,7 @@ CartShape cart_shape(const DevNet &N, int occ) {
         cudaGetLastError();
         return sh;
     }
-    const long budget = ((long)smem_sm / by_regs - 4096) / 8;
+    const long budget = stage_budget(smem_sm, by_regs, occ == 8, most);
     sh.cap = (int)(std::max<long>(0, std::min<long>(want, budget)) & ~1l);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 128, (size_t)sh.cap * sizeof(double)) !=
             cudaSuccess || per_sm < 1) {

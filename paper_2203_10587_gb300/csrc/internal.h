@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <functional>
 #include <string>
@@ -77,6 +78,7 @@ struct DevNet {
     int nb, nl, ng, n, m, nslot;
     int64_t nnzJ, nnzJg, nnzH, hpg;          // hpg: H position of (Pg_0, Pg_0)
     int jP_end, jQ_end, hA_end, hM_end;      // ends of the four row blocks of the bus rows
+    int stage_cap_most[4];                   // stage_cap_rows without the largest sixteenth of the tiles
     int stage_cap_rows[4];                   // shared-memory doubles of a bus tile of 32/64/128/256
     int stage_cap_all[4];                    // buses: its row segments, or components plus rows
     int stage_cap_bulk[4];                   // ... or its whole records plus rows
@@ -237,6 +239,34 @@ int state_allow_smem();
 int launch_eval_state(const DevNet &net, const EvalReq &req, int nt, size_t smem, void *stream);
 
 constexpr int kStageMaxDoubles = 9216;   // 72 KB
+
+// Doubles of shared memory that each of `ctas` resident CTAs of an SM may stage its bus tiles in;
+// most: what all but a sixteenth of the tiles need for their rows.
+//
+// The SM's 256 KB are divided between shared memory and L1 in steps, the one for 228 KB of shared
+// memory leaving L1 28 KB, 196 KB 60, 164 KB 92, and the items' gathers (voltages, multipliers,
+// tables) live in L1.  One 64-bus tile of 22,016 bytes in place of 21,952 put eight CTAs over 196 KB
+// and took 10,000 buses x 64 states from 261 to 304 us.  So: 164 KB where all but a sixteenth of
+// the tiles fit, else 196 (us, by limits of 228, 196, 164, 132 and 100 KB):
+//   10,000 x 64    64 threads    304 261 258 260 270     slot-parallel 311 289 289
+//                  bulk          270 261 265 272 275     multi-kernel  419 332 331
+//   2,000 x 512    64 threads    413 413 411 415 432     slot-parallel 493 471 471
+//                  bulk          422 418 425 436 436     multi-kernel  670 533 536
+//   2,000 x 301 of 6,000 branches    128 threads 825 620 655    bulk 799 643 657
+//   cartesian      2,000 x 512 485 484 485 487; 10,000 x 64 319 320 311 311; 2,000 x 200 of 6,000
+//                  branches 615 441 461 452
+// With the compiler's registers (few_warps: occupancy 8) the staged rows and records count for more
+// than L1 (bulk, 10,000 x 1: 24.9 26.9 26.8; 2,000 x 16: 33.4 36.3 35.7): no limit there.
+inline long stage_budget(long smem_per_sm, int ctas, bool few_warps, int most) {
+    if (ctas < 1) ctas = 1;
+    long doubles = (smem_per_sm / ctas - 4096) / 8;
+    if (!few_warps) {
+        // a CTA's share of `kb`, less its static part and the 1 KB the system takes
+        auto within = [&](long kb) { return (((kb << 10) / ctas & ~127l) - 3136) / 8; };
+        doubles = std::min(doubles, most <= within(164) ? within(164) : within(196));
+    }
+    return std::max(0l, doubles);
+}
 // The persistent schedule's ring slot of one state: NCOMP x nslot doubles of branch-end records,
 // then the kObjLanes partial sums of the state's objective (256 virtual lanes).
 constexpr int kObjLanes = 256;
