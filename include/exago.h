@@ -462,10 +462,8 @@ exago_status exago_eval_profile(exago_net_t net, const exago_batch *batch, doubl
  *             wait times out; the launch still ends and exago_net_check reports it.
  *   tile_group  persistent: tiles of one kind and state per work item (1 to 4; 0 = 1), which
  *             divides the items' claims, waits and signals by that number.
- *   tiling    persistent: EXAGO_TILING_THREAD: branch per thread -- each thread of a tile takes
- *             its own branch (bus) of one state.  EXAGO_TILING_DEFAULT: the same, but branch per
- *             warp for large batches of meshed grids (2.5 to 3 branches a bus or more) when no
- *             other field of the configuration is set.  EXAGO_TILING_WARP: branch per warp
+ *   tiling    persistent: EXAGO_TILING_DEFAULT / THREAD: branch per thread -- each thread of a
+ *             tile takes its own branch (bus) of one state.  EXAGO_TILING_WARP: branch per warp
  *             -- each warp takes one branch (bus) and its 32 lanes take 32 consecutive states,
  *             so every lane of a warp walks a bus of the same degree; blocks of 128 (0 = 128)
  *             or 64 threads, occupancy 8 or 16, tile_group branches (buses) per warp and work item,

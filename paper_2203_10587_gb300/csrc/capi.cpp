@@ -353,29 +353,6 @@ bool untouched(const exago_config &c) {
            !c.tile_group && !c.tiling;
 }
 
-// Whether an untouched configuration runs branch-per-warp tiles: on meshed grids, where a
-// per-thread bus tile's warps run to their highest-degree bus and its rows outgrow the staging.
-// Measured on GB300, per thread against per warp (us; the second pair with generator masks):
-//   branches a bus  grid, states        without masks      with masks
-//   1.35            2,000 x 512         416 against 468    436 against 556
-//   2.0             2,000 x 512         684 against 663    710 against 722
-//   2.5             2,000 x 100         209 against 207    216 against 239
-//   2.5             2,000 x 301         573 against 499    590 against 533
-//   3.0             2,000 x 32          119 against  95    122 against 116
-//   3.0             2,000 x 301         780 against 587    799 against 623
-//   3.0             500 x 64             65 against  70     65 against  78
-//   3.0             500 x 100           100 against  85    104 against  93
-//   3.4             118 x 100            48 against  57     49 against  63
-//   3.4             118 x 301            97 against  84    101 against  92
-// so: three branches a bus and 120,000 branch items, or two and a half and a million; fewer than 32
-// states leave lanes idle.
-bool prefer_warp_tiles(const exago_net *net, const exago_config &c, int B) {
-    if (!untouched(c)) return false;
-    const double nl = net->plan.nl, items = nl * B;
-    if (B < 32) return false;
-    return (nl >= 3.0 * net->plan.nb && items >= 1.2e5) || (nl >= 2.5 * net->plan.nb && items >= 1e6);
-}
-
 Resolved resolve(exago_net *net, int B) {
     exago_config c = net->cfg;
     if (c.schedule == EXAGO_SCHED_AUTO) {
@@ -411,7 +388,7 @@ Resolved resolve(exago_net *net, int B) {
     r.spin_limit = c.spin_limit > 0 ? c.spin_limit : kDefaultSpinLimit;
     r.force_timeout = c.test_force_timeout ? 1 : 0;
     r.group = c.tile_group >= 1 && c.tile_group <= 4 ? c.tile_group : 1;
-    if (pers && (c.tiling == EXAGO_TILING_WARP || prefer_warp_tiles(net, c, B))) {
+    if (pers && c.tiling == EXAGO_TILING_WARP) {
         // warp-tiled: blocks of 128 (default) or 64 threads, no record staging; the lag and the
         // ring count groups of 32 states.  By default bus items trail by the groups the resident
         // CTAs hold in branch work plus two, and the ring holds two lags (measured on 2000 buses
