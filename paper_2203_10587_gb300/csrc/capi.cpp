@@ -427,7 +427,7 @@ Resolved resolve(exago_net *net, int B) {
     if (pers && untouched(net->cfg) && !net->tuned.count(B)) {
         // One wave of items: warps are few, so a block with all the registers it wants (12 warps an SM)
         // and its records in one bulk copy is faster (us, default against this: 10,000 buses x 1
-        // state 27.1, 25.1; x 4 41.2, 35.0; 2,000 x 1 24.7, 22.6; x 16 37.3, 33.5; 500 x 64 36.6, 32.9).
+        // state 27.1, 25.0; x 4 37.2, 35.0; 2,000 x 1 24.7, 22.6; x 16 36.6, 33.5; 500 x 64 36.6, 32.9).
         // A little over a wave it loses (1,000 x 64 44.4, 46.9; 4,000 x 16 45.2, 55.6).
         const double items = (double)B * ((std::max(net->plan.nl, net->plan.nb) + 63) / 64);
         if (items <= (double)net->sm_count * occupancy(net, true, 64, 8, 0)) {
@@ -473,7 +473,9 @@ StateBlock state_block(const exago_net *net, int B) {
         return rec + *cap * sizeof(double);
     };
     // Estimated times (us), fitted to 9 grids of 30 to 900 buses x 1 to 1,024 states (all outputs):
-    //   persistent            24 + 0.34 per 1,000 branch items;
+    //   persistent            24 + 0.34 per 1,000 branch items; a block a state being at most one
+    //                         wave, and so its items, no more than 26.5 + 0.0125 a 64-branch item (707
+    //                         x 106 42.5, where 256 threads a state took 49.3; 612 x 112 39.4, 41.1);
     //   256 threads a state   12 + 0.052 a branch for one block an SM; two resident blocks of a
     //                         further wave take 0.72 of one's time each;
     //   64 threads a state    7.5 + 0.14 a branch, the blocks of an SM overlapping (up to 160
@@ -487,7 +489,9 @@ StateBlock state_block(const exago_net *net, int B) {
     const size_t b64 = smem_of(64, &cap64), b256 = smem_of(256, &cap256);
     const bool two = 2 * (b256 + 3072) <= (size_t)net->smem_per_sm;   // with the static part
     const double waves = std::ceil(per_sm);
-    const double pers = 24.0 + 0.34e-3 * nl * B;
+    const double items = (double)B * ((std::max(net->plan.nl, net->plan.nb) + 63) / 64);
+    double pers = 24.0 + 0.34e-3 * nl * B;
+    if (waves <= 1.0 && items <= 8.4 * net->sm_count) pers = std::min(pers, 26.5 + 0.0125 * items);
     const double t256 = (12.0 + 0.052 * nl) * (waves <= 1.0 ? 1.0 : two ? 0.72 * waves : waves);
     const double t64 = nl > 160 ? 1e30 : (7.5 + 0.14 * nl) * std::max(1.0, 0.6 + 0.22 * per_sm);
     const double t512 = waves > 1.0 ? 1e30 : nl <= 64 ? 12.5 : nl > 256 && nl <= 512 ? 10.0 + 0.05 * nl : 1e30;
