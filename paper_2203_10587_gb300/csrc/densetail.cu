@@ -26,6 +26,38 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// ---- balanced columns ----------------------------------------------------------------------------
+
+// Column k of a panel is split as G_ik = F_ik 2^-c and H_jk = L_jk 2^c (LU: U'_jk 2^c), c half the
+// exponent of its pivot d_k, here from the pivot's reciprocal (0 where that is zero, subnormal or not
+// finite).  The scales cancel in the products.  With F = L D both operands are then about
+// L_ik sqrt|d_k|, whose squares sum to the matrix's own diagonal entry at most (but for growth), so
+// the split's errors are relative to sqrt|a_ii a_jj| as those of an elimination in FP64 are,
+// whatever the scales of the variables.  Unscaled, the largest entries of a row of F and of one of L
+// lie in different columns when pivots differ, as barrier terms make them near convergence: with
+// barrier terms over 4, 8 and 12 decades the KKT step was 20, 45 and 26 times as far off as an
+// elimination in FP64 for 150 buses of 450 branches (7, 4 and 7 for 100 of 260), balanced it is 1.2, 0.7
+// and 0.4 (1.3, 1.1, 0.4).  2,000 buses x 512 states take 15.50 ms unscaled, 15.55 balanced.
+__device__ __forceinline__ int half_exp(double r) {
+    const int f = (__double2hiint(r) >> 20) & 0x7ff;
+    return (unsigned)(f - 1) < 2046u ? (1023 - f) >> 1 : 0;
+}
+
+// v 2^c, |c| <= 1024, by moving the exponent field (a multiplication takes the FP64 pipe 64 cycles a
+// warp); false, and v as it was, where either end is not a normal number.
+__device__ __forceinline__ bool scale_normal(double &v, int c) {
+    const int hi = __double2hiint(v), f = (hi >> 20) & 0x7ff;
+    if (!((hi << 1) | __double2loint(v))) return true;   // zero
+    if ((unsigned)(f - 1) >= 2046u || (unsigned)(f + c - 1) >= 2046u) return false;
+    v = __hiloint2double(hi + c * (1 << 20), __double2loint(v));
+    return true;
+}
+__device__ __forceinline__ double scale(double v, int c) {
+    if (scale_normal(v, c)) return v;
+    const int h = c / 2;
+    return v * __hiloint2double((1023 + h) << 20, 0) * __hiloint2double((1023 + c - h) << 20, 0);
+}
+
 // ---- digits --------------------------------------------------------------------------------------
 
 // Exponent field of |v| (subnormals and zero: 1).
@@ -294,7 +326,8 @@ __device__ __forceinline__ size_t digit_at(int P, int K, int s, int I) {
 }
 
 // One tile of 128 rows (DIAG: the panel's own 64) of panel J, one block per (tile, state).
-// MODE 0: F and L (SYM); 1: F alone (LU, lower side); 2: U' from G = U' D' (LU, upper side).
+// MODE 0: F and L (SYM); 1: F alone (LU, lower side); 2: U' from U' D' (LU, upper side).  Targets are
+// T 2^-c from the start, and what is left in their place is G = F 2^-c (MODE 2: H = U' 2^c).
 // What bounds it: the 8,192 targets' integer joins and two FP64-pipe instructions each, beside 2.4
 // us of tensor work a 64-deep step; one block per SM (172 KB of digits), 16 warps that finish
 // products beside one that issues copies and MMAs.  The columns go in two halves of 32, each with
@@ -311,12 +344,19 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_dead;
     __shared__ int s_eb[2][64], s_em[64 / kCols][128];
+    __shared__ __align__(16) int s_c[64];        // the panel's columns' exponents (half_exp)
+    __shared__ __align__(16) double s_hg[64];    // H / G: the pivots' reciprocals, scaled by 2^2c
     char *sA = (char *)(((uintptr_t)raw + 1023) & ~(uintptr_t)1023), *sB = sA + kSmemA;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const size_t st = blockIdx.y;
     const int n = A.n, P = A.P, J = A.J;
     const int I0 = DIAG ? J : J + 1 + 2 * (int)blockIdx.x;   // first 64-row tile
     const int tiles = DIAG ? 1 : min(2, P - I0);
+    if (!DIAG && tid < 64) {
+        const double r = __ldcg(A.dinv + st * n + 64 * J + tid);
+        s_c[tid] = half_exp(r);
+        s_hg[tid] = scale(r, 2 * s_c[tid]);
+    }
     if (tid == 0) {
         mbar_init(&bar_full, 1);
         for (int h = 0; h < 2; h++) {
@@ -393,10 +433,22 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
         double acc[kCols] = {};
 #pragma unroll
         for (int c = 0; c < NC; c++) acc[c] = live ? __ldcg(Dp + (size_t)c * ld) : 0.0;
+        if (!DIAG) {   // T 2^-c, while the first operands are copied
+            bool normal = true;
+#pragma unroll
+            for (int c = 0; c < kCols; c++) normal &= scale_normal(acc[c], -s_c[c0 + c]);
+            if (!normal) {   // all of them again, one after the other
+#pragma unroll 1
+                for (int c = 0; c < kCols; c++) {
+#pragma unroll
+                    for (int i = 1; i < kCols; i++) acc[i - 1] = acc[i];
+                    acc[kCols - 1] = scale(__ldcg(Dp + (size_t)c * ld), -s_c[c0 + c]);
+                }
+            }
+        }
         const int *xa = A.xa + st * (size_t)P * n, *xb = A.xb + st * (size_t)P * n;
-        const double *dinv = A.dinv + st * n + 64 * J + c0;
-        // steps K < J: the products of the panels before; J: the targets times the inverse, F_IJ
-        // (MODE 2: U'); J + 1: its digits kept for the panels to come; J + 2: L_IJ's (MODE 0)
+        // steps K < J: the products of the panels before; J: the targets times the inverse, G_IJ
+        // (MODE 2: H_IJ); J + 1: its digits kept for the panels to come; J + 2: H_IJ's (MODE 0)
         const int steps = DIAG ? J : J + (MODE == 0 ? 3 : 2);
         const bool mine = (tid & (kEpi / 2 - 1)) < 32;    // one warp of a half keeps its columns' exponents
         const int col = 32 * half + lane;
@@ -404,7 +456,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
         for (int K = 0; K < steps; K++) {
             int ea = 0;
             if (DIAG || K < J) {
-                if (mine) s_eb[K & 1][col] = __ldcg(xb + (size_t)K * n + 64 * J + col);
+                if (mine) s_eb[K & 1][col] = __ldcg(xb + (size_t)K * n + 64 * J + col) - (DIAG ? 0 : s_c[col]);
                 if (live) ea = __ldcg(xa + (size_t)K * n + grow);
                 half_sync(half);
             } else {
@@ -439,7 +491,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
                 if (!DIAG && K == J) {
                     if (MODE == 2)
 #pragma unroll
-                        for (int c = 0; c < kCols; c++) acc[c] *= __ldcg(dinv + c);
+                        for (int c = 0; c < kCols; c++) acc[c] *= s_hg[c0 + c];
                     if (live)
 #pragma unroll
                         for (int c = 0; c < kCols; c++) Dp[(size_t)c * ld] = acc[c];
@@ -458,7 +510,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_dt_update(const UpdateArgs A
                 }
                 if (MODE == 0 && !second)
 #pragma unroll
-                    for (int c = 0; c < kCols; c++) acc[c] *= __ldcg(dinv + c);
+                    for (int c = 0; c < kCols; c++) acc[c] *= s_hg[c0 + c];
                 epi_sync();
             }
         }
@@ -478,8 +530,8 @@ constexpr int kPitch = 65;   // doubles per column in shared memory: rows of a c
                              // of a row both spread over the banks
 
 // Digits of the 64 x 64 unit lower triangular X (shared memory, X[k * kPitch + row] below the diagonal)
-// with one exponent per row.
-__device__ __forceinline__ void panel_digits(const double *X, char *out, int *xout) {
+// with one exponent per row, as X_jk 2^(c_k - c_j): it takes T 2^-c to G.
+__device__ __forceinline__ void panel_digits(const double *X, const int *c, char *out, int *xout) {
     for (int it = threadIdx.x; it < 512; it += kFacThreads) {
         const int row = it >> 3, grp = it & 7;
         double v[8];
@@ -487,7 +539,7 @@ __device__ __forceinline__ void panel_digits(const double *X, char *out, int *xo
 #pragma unroll
         for (int k = 0; k < 8; k++) {
             const int col = 8 * grp + k;
-            v[k] = row > col ? X[col * kPitch + row] : row == col ? 1.0 : 0.0;
+            v[k] = row > col ? scale(X[col * kPitch + row], c[col] - c[row]) : row == col ? 1.0 : 0.0;
             E = max(E, exp_field(v[k]));
         }
         for (int h = 1; h < 8; h <<= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, h));
@@ -567,6 +619,7 @@ __global__ void __launch_bounds__(kFacThreads, 4) k_dt_factor(int n, int J, doub
     extern __shared__ double sm[];
     double *Ls = sm;   // L by columns, Ls[k * kPitch + i], i > k; LU: row k of D U at Ls[j * kPitch + k]
     __shared__ double s_f[2][64], s_d[64], s_r[64];
+    __shared__ int s_c[64];   // the columns' exponents (half_exp)
     __shared__ unsigned long long s_max[64];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const size_t st = blockIdx.x;
@@ -646,6 +699,7 @@ __global__ void __launch_bounds__(kFacThreads, 4) k_dt_factor(int n, int J, doub
     __syncthreads();
     if (tid < 64) {
         dinv[st * n + 64 * J + tid] = s_r[tid];
+        s_c[tid] = half_exp(s_r[tid]);
         unsigned long long a = 0;
         for (int h = 0; h < BS; h++) a = max(a, s_max[tid / BS * BS + h]);
         const double d = s_d[tid];
@@ -672,7 +726,7 @@ __global__ void __launch_bounds__(kFacThreads, 4) k_dt_factor(int n, int J, doub
             out[(size_t)j * ld + lane + 32] = hi[c];
         }
         __syncthreads();
-        panel_digits(Ls, digits + st * kDigits * kTile, exps + st * 64);
+        panel_digits(Ls, s_c, digits + st * kDigits * kTile, exps + st * 64);
     };
     unit_inverse<false>(Ls, warp, lane, lo, hi);
     finish(Dp, linv, line);
@@ -702,14 +756,16 @@ __device__ __forceinline__ double sum8(double *a, int lane) {
     return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
 }
 
-// Both sweeps of one state's tail.  Forward, per panel: z = L^-1 r, the rows below lose F D^-1 z;
-// backward: the panel's unknowns lose U's (or D^-1 F's) part, then L^-T (U^-1).
+// Both sweeps of one state's tail.  Forward, per panel: z = D^-1 L^-1 r, the rows below lose F z; backward:
+// the panel's unknowns lose U's (or D^-1 F's) part, then L^-T (U^-1).  Below the panels' squares D holds
+// G = F 2^-c and V H = U' 2^c (half_exp).
 template <bool SYM>
 __global__ void __launch_bounds__(kSolThreads) k_dt_solve(int n, int nreal, int B, const double *D,
                                                           const double *V, size_t dstride,
                                                           const double *dinv, double *x0) {
     extern __shared__ double sx[];               // [n] the vector, then [4][64] partial sums
     double *part = sx + n;
+    __shared__ double zs[64];                    // z 2^c
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const size_t st = blockIdx.x;
     const double *Db = D + st * dstride, *Vb = SYM ? Db : V + st * dstride;
@@ -725,9 +781,12 @@ __global__ void __launch_bounds__(kSolThreads) k_dt_solve(int n, int nreal, int 
         for (int k = 16 * q4; k < 16 * q4 + 16; k++) a = fma(__ldg(Dp + (size_t)k * ld + r64), sx[j0 + k], a);
         part[q4 * 64 + r64] = a;
         __syncthreads();
-        if (tid < 64)
-            sx[j0 + tid] = ((part[tid] + part[64 + tid]) + (part[128 + tid] + part[192 + tid])) *
-                           __ldg(di + j0 + tid);
+        if (tid < 64) {
+            const double r = __ldg(di + j0 + tid);
+            const double z = ((part[tid] + part[64 + tid]) + (part[128 + tid] + part[192 + tid])) * r;
+            sx[j0 + tid] = z;
+            zs[tid] = scale(z, half_exp(r));
+        }
         __syncthreads();
         // four sums of 16 terms, then one subtraction: shorter chains, and fewer roundings at the
         // size of the target
@@ -737,7 +796,7 @@ __global__ void __launch_bounds__(kSolThreads) k_dt_solve(int n, int nreal, int 
             for (int k = 0; k < 64; k += 4)
 #pragma unroll
                 for (int h = 0; h < 4; h++)
-                    a[h] = fma(__ldg(Dp + (size_t)(k + h) * ld + i), sx[j0 + k + h], a[h]);
+                    a[h] = fma(__ldg(Dp + (size_t)(k + h) * ld + i), zs[k + h], a[h]);
             sx[j0 + i] -= (a[0] + a[1]) + (a[2] + a[3]);
         }
         __syncthreads();
@@ -757,7 +816,11 @@ __global__ void __launch_bounds__(kSolThreads) k_dt_solve(int n, int nreal, int 
             }
             const double t = sum8(a, lane);
             const int c = 8 * warp + (lane >> 2);
-            if ((lane & 3) == 0) part[c] = SYM ? fma(-t, __ldg(di + j0 + c), sx[j0 + c]) : sx[j0 + c] - t;
+            if ((lane & 3) == 0) {
+                const double r = __ldg(di + j0 + c);
+                const int e = half_exp(r);
+                part[c] = SYM ? fma(-t, scale(r, e), sx[j0 + c]) : sx[j0 + c] - scale(t, -e);
+            }
         }
         __syncthreads();
         // x_k = sum_i X[i][k] w_i, X = L^-1 (SYM) or U'^-1: column k of the panel's inverse

@@ -4,12 +4,15 @@
 //
 // On bus graphs a minimum-degree order ends in a clique that holds almost all of the work: on the
 // 2,000-bus grid the last 192 columns hold 95% of the block products (1.02 of 1.07 million per
-// state) and 179 of the 190 levels.  Those products run here on the tensor cores, exactly split:
+// state) and 179 of the 190 levels.  Those products run here on the tensor cores, in 62-bit fixed point:
 //
-//   * A panel of 64 scalar columns of F = L D (and of L, or U' for LU) is kept, besides its FP64
-//     values, as 7 "digits" per value: with 2^e above every magnitude of a row's 64 values, each
-//     value is X 2^(e-62), X a 62-bit integer written in base 512 with digits in [-256, 256], so
-//     every digit is exact in bf16.
+//   * A panel of 64 scalar columns of F = L D (and of L, or U' for LU) is kept as G = F 2^-c and
+//     H = L 2^c, the columns balanced by powers of two (half_exp), G in FP64 and both as 7 "digits"
+//     per value: with 2^e above every magnitude of a row's 64 values, each value is X 2^(e-62), X a
+//     62-bit integer written in base 512 with digits in [-256, 256], so every digit is exact in
+//     bf16.  A value below 2^-9 of its row's largest loses its lowest bits; the error of a product
+//     is then 2^-61 of the rows' largest values, relative to sqrt|a_ii a_jj| as that of an FP64
+//     elimination is (2^-53 of the terms' sum there).
 //   * The product of two such rows is sum over digit pairs (s, t) of 2^(-9(s+t)) D_st, D_st a sum
 //     of 64 products of integers of at most 2^16.  The 28 pairs with s + t <= 6 are multiplied by
 //     tcgen05.mma into 7 FP32 accumulators in TMEM, one per s + t.  The sums with s + t <= 3 stay
@@ -24,7 +27,7 @@
 // together, 2,000 buses x 512 states: KKT step 96.3 to 15.5 ms, power-flow step 37.3 to 7.8 ms;
 // 200 buses x 37 states, where the 190 levels' launches went instead: 1,442 to 493 us.  Mean error
 // of the step against extended precision, before and after: 4.29e-15 and 4.31e-15 (2,000 buses),
-// 5.9e-16 and 6.1e-16 (200).
+// 5.9e-16 and 6.1e-16 (200); with barrier terms over many decades see half_exp.
 //
 // Per panel J of 64 columns, for every state:
 //   k_dt_update<diag>  T_JJ -= sum_{K<J} F_JK L_JK'
@@ -32,8 +35,8 @@
 //                      the 4 x 4 (2 x 2) pivot blocks in order -- and the inverse of its unit
 //                      triangle(s)
 //   k_dt_update<rows>  for the 128-row tiles below: T_IJ -= sum_{K<J} F_IK L_JK', then
-//                      F_IJ = T_IJ L_JJ^-T by the same digit product with the inverse, and the
-//                      digits of F_IJ and of L_IJ = F_IJ D_J^-1
+//                      F_IJ = T_IJ L_JJ^-T by the same digit product with the inverse (all of it
+//                      with the columns balanced: G), and the digits of G_IJ and of H_IJ
 // and k_dt_solve does both triangular sweeps of the tail.
 #pragma once
 
