@@ -167,17 +167,17 @@ __device__ __forceinline__ End end_terms(double Gss, double Bss, double Gss2, do
                                          double A, double C, double Vu, double Vv, double Vu2,
                                          double VV, M &mul) {
     End e;
-    mul.need(A);
-    mul.need(C);
-    e.qa = mul(VV, A);             //  Vu Vv A
-    e.pa = -mul(VV, C);            // -Vu Vv C
+    mul.need_or_zero(A);
+    mul.need_or_zero(C);
+    e.qa = mul.or_zero(VV, A);     //  Vu Vv A
+    e.pa = -mul.or_zero(VV, C);    // -Vu Vv C
     e.P = fma(Gss, Vu2, e.qa);
     e.Q = fma(-Bss, Vu2, -e.pa);
     if (DERIV) {
-        e.pv = mul(Vu, A);
-        e.qv = mul(Vu, C);
-        e.pu = fma(Gss2, Vu, mul(Vv, A));
-        e.qu = fma(-Bss2, Vu, mul(Vv, C));
+        e.pv = mul.or_zero(Vu, A);
+        e.qv = mul.or_zero(Vu, C);
+        e.pu = fma(Gss2, Vu, mul.or_zero(Vv, A));
+        e.qu = fma(-Bss2, Vu, mul.or_zero(Vv, C));
     }
     return e;
 }
@@ -200,19 +200,19 @@ __device__ __forceinline__ EndHess end_hess(const End &e, double Gss2, double Bs
                                             double C, double K, double Vu, double Vv,
                                             double lamP, double lamQ, double mu, M &mul) {
     EndHess h;
-    mul.need(e.pu);
-    mul.need(e.qu);
+    mul.need_or_zero(e.pu);
+    mul.need_or_zero(e.qu);
     const double mu2 = twice(mu);
     const double wP = fma(mu2, e.P, lamP);
     const double wQ = fma(mu2, e.Q, lamQ);
     h.W1 = fma(wP, A, wQ * C);
     h.W2 = fma(wQ, A, -(wP * C));
-    const double E = fma(A, e.qu, -mul(C, e.pu));
-    const double F = fma(e.pu, A, mul(e.qu, C));
+    const double E = fma(A, e.qu, -mul.or_zero(C, e.pu));
+    const double F = fma(e.pu, A, mul.or_zero(e.qu, C));
     h.tK = mu2 * K;
     const double mu2Vu = mu2 * Vu;
     h.hau = Vv * fma(mu2Vu, E, h.W2);             // 2 mu Vu Vv E + Vv W2
-    const double S = fma(e.pu, e.pu, mul(e.qu, e.qu));
+    const double S = fma(e.pu, e.pu, mul.or_zero(e.qu, e.qu));
     h.huu = fma(mu2, S, fma(wP, Gss2, -(wQ * Bss2)));
     h.huv = fma(mu2Vu, F, h.W1);
     return h;

@@ -46,17 +46,38 @@ __device__ __forceinline__ bool mul_window(double x) {
     return ((uint32_t)__double2hiint(x) << 1) - (768u << 21) < (512u << 21);
 }
 
+__device__ __forceinline__ bool is_zero(double x) {
+    return (((uint32_t)__double2hiint(x) << 1) | (uint32_t)__double2loint(x)) == 0;
+}
+
+// x y, correctly rounded, for x and y in mul_window or zero: what int_mul gives, or a zero of the
+// product's sign.
+__device__ __forceinline__ double int_mul_zero(double x, double y) {
+    const double p = int_mul(x, y);
+    const int sign = (__double2hiint(x) ^ __double2hiint(y)) & (int)0x80000000;
+    return is_zero(x) || is_zero(y) ? __hiloint2double(sign, 0) : p;
+}
+
 // How an item multiplies.  INT: products whose operands are ordinary values (voltages, flows and
-// their derivatives, never multipliers or sin th, which may be zero) go to the integer pipe;
-// need() notes an operand outside the window, and the item is then computed again with INT = false.
+// their derivatives, never multipliers or sin th) go to the integer pipe; need() notes an operand
+// outside the window, and the item is then computed again with INT = false.  Operands that are exactly
+// zero in ordinary states (of a lossless branch without an angle across it the conductance terms)
+// are noted by need_or_zero() and multiplied by or_zero(): computed twice, they took every warp that
+// held one such branch through both paths.
 template <bool INT>
 struct Mul {
     bool ok = true;
     __device__ __forceinline__ double operator()(double x, double y) const {
         return INT ? int_mul(x, y) : x * y;
     }
+    __device__ __forceinline__ double or_zero(double x, double y) const {
+        return INT ? int_mul_zero(x, y) : x * y;
+    }
     __device__ __forceinline__ void need(double x) {
         if (INT) ok = ok && mul_window(x);
+    }
+    __device__ __forceinline__ void need_or_zero(double x) {
+        if (INT) ok = ok && (mul_window(x) || is_zero(x));
     }
 };
 
