@@ -505,7 +505,9 @@ exago_status exago_net_get_config(exago_net_t net, int B, exago_config *cfg);
  * variants (branch per warp: block 64 / 128, occupancy 8 / 16, 1 or 2 branches per warp and
  * item), on this batch, `reps` evaluations each after one warm-up, on batch->stream, and records the
  * fastest for batches of this size (used by EXAGO_SCHED_AUTO).  Outputs are written as by
- * exago_eval_all.  *best (may be NULL) receives the choice.
+ * exago_eval_all.  *best (may be NULL) receives the choice.  Where the automatic rule has one block
+ * per state for this batch, that is timed too, and an untouched configuration keeps it if it was
+ * faster than the choice (*best and exago_net_get_config return the choice all the same).
  */
 exago_status exago_net_autotune(exago_net_t net, const exago_batch *batch, double *f, double *grad,
                                 double *gh, double *jval, double *hval, int reps,
