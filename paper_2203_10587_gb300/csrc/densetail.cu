@@ -589,28 +589,15 @@ __device__ __forceinline__ unsigned long long mag(double v) {
     return u > 0x7ff0000000000000ull ? 0 : u;
 }
 
-__device__ __noinline__ double reciprocal_any(double d) { return 1.0 / d; }
-
-// 1 / d.  The hardware's approximation r0 (rcp.approx.ftz.f64, about 20 bits) and one step of the
-// third-order Householder iteration, r0 + r0 (e + e^2) with e = 1 - d r0: three dependent FP64
-// instructions on the chain of the 64 pivots, in place of the division's ten or so.  Zero,
-// subnormal, huge and non-finite d, where r0 or e would not be ordinary, are divided.
-__device__ __forceinline__ double reciprocal(double d) {
-    const unsigned f = ((unsigned)__double2hiint(d) >> 20) & 0x7ff;
-    if (f - 64u > 1900u) return reciprocal_any(d);
-    double r0;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
-    const double e = fma(-d, r0, 1.0);
-    return fma(r0, fma(e, e, e), r0);
-}
-
 // L D L' (or L D U) of the panel's 64 x 64 diagonal block without pivoting, one block per state;
 // then the inverses of L (and of U'), as digits for the rows below and in FP64, in place of the
 // block, for the sweeps.  Warp w holds columns w, w + 8, .. in registers, a lane rows lane and
 // lane + 32.  Step k subtracts column k's part from the columns after it; the warp that holds column
 // k + 1 does that one first, and its pivot, reciprocal and publication, while the others work.
 // Bound by the FP64 pipe (about 5,000 warp instructions of 64 cycles over four pipes) and, for
-// few states, by the chain of pivots: 192 us for 512 states (290 before the look-ahead), 72 for 37.
+// few states, by the chain of pivots: 192 us for 512 states (290 before the look-ahead), 76 for 37.
+// The pivots are divided, as everywhere else: a step from the hardware's approximation was 3 us
+// shorter on 37 states and up to 1 ulp off.
 template <bool SYM, int BS>
 __global__ void __launch_bounds__(kFacThreads, 4) k_dt_factor(int n, int J, double *D, double *V,
                                                            size_t dstride, double *dinv, char *linv,
@@ -642,7 +629,7 @@ __global__ void __launch_bounds__(kFacThreads, 4) k_dt_factor(int n, int J, doub
     // column k = warp + 8 c is final: its pivot, and the column for the other warps
     auto publish = [&](int c, int k) {
         const double d = __shfl_sync(0xffffffffu, c < 4 ? lo[c] : hi[c], k & 31);
-        const double r = reciprocal(d);
+        const double r = 1.0 / d;
         const double fl = lane > k ? lo[c] : 0.0, fh = lane + 32 > k ? hi[c] : 0.0;
         s_f[k & 1][lane] = fl;
         s_f[k & 1][lane + 32] = fh;
