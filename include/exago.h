@@ -616,15 +616,20 @@ exago_status exago_serve_drive(exago_server_t server, const exago_serve_client *
  *                         the elimination tree, and FP64 flops of one state's factor and solve.
  *   exago_kkt_workspace_size  scratch bytes for B states (two factor arrays of 16 x 8 B x B per
  *                         factor block, one without the dense last columns, whose panels and
- *                         split operands come beside them; the reduced vectors and counters).
+ *                         split operands, up to 8 GB of them, come beside them; the reduced vectors
+ *                         and counters): 2,000 buses x 512 states 8.3 GB.
  *   exago_kkt_solve       DEVICE pointers, row-major per state: jval [B][nnzJ], hval [B][nnzH],
  *                         dx [B][n], dc [B][m] (> 0), rhs [B][n + m]; sol [B][n + m] receives
  *                         [dx; dlam].  inertia [B][2] (or NULL) receives the number of negative
  *                         pivots of the whole factorisation (m for a correct interior-point step)
  *                         and of pivots below 1e-13 of their block (0 unless K is numerically
- *                         singular without pivoting).  workspace: at least exago_kkt_workspace_size
+ *                         singular without pivoting).  workspace: exago_kkt_workspace_size
  *                         bytes, 256-byte aligned, or NULL for the handle's own (grown on demand;
  *                         a growth synchronises the device; calls using it must be ordered).
+ *                         A smaller one is taken if it holds two whole factor arrays, the vectors
+ *                         and counters, each rounded up to 256 bytes, and so is the handle's own
+ *                         where the device has no room for more: the last columns are then factored as the
+ *                         others are, which takes longer and rounds differently.
  *                         Asynchronous on `stream`.  EINVAL for null arguments or B too large.
  */
 typedef struct exago_kkt *exago_kkt_t;
@@ -654,7 +659,8 @@ exago_status exago_kkt_solve(exago_kkt_t kkt, int B, const double *jval, const d
  *                            columns as in exago_kkt_workspace_size, lower and upper, vectors).
  *   exago_pf_step            x_new [B][n] (DEVICE; may equal batch->x) = x + d, Pg and Qg copied;
  *                            mismatch [B] (or NULL) = max |g_pf(x)| before the step.
- *                            batch->workspace: at least exago_pf_workspace_size bytes, or NULL for
+ *                            batch->workspace: exago_pf_workspace_size bytes (or fewer, as for
+ *                            exago_kkt_solve: g, J and four whole factor arrays), or NULL for
  *                            the handle's own (grown on demand, synchronising the device; calls
  *                            using it must be ordered); the evaluation inside uses the net's
  *                            internal workspace.  batch->lambda is ignored.  Asynchronous on

@@ -749,8 +749,28 @@ int launch_block_solve(const DevSym &S, int B, const double *T, const double *L,
     return (int)cudaGetLastError();
 }
 
-int upload_block_sym(const BlockSym &S, DevSym &D, std::vector<void *> &allocs) {
-    D = DevSym();
+exago_status grow_workspace(void **ws, size_t *bytes, size_t need, size_t least, const char *what) {
+    if (*bytes >= need) return EXAGO_OK;
+    size_t room = 0, total = 0;
+    if (least < need && cudaMemGetInfo(&room, &total) == cudaSuccess && room + *bytes < need) need = least;
+    if (*bytes >= need) return EXAGO_OK;
+    if (*ws) {
+        cudaError_t e = cudaDeviceSynchronize();
+        if (e != cudaSuccess) return set_last_error(EXAGO_ECUDA, cudaGetErrorString(e));
+        cudaFree(*ws);
+        *ws = nullptr;
+        *bytes = 0;
+    }
+    cudaError_t e = dev_malloc(ws, need);
+    if (e != cudaSuccess) {
+        *ws = nullptr;
+        return set_last_error(e == cudaErrorMemoryAllocation ? EXAGO_ENOMEM : EXAGO_ECUDA, what);
+    }
+    *bytes = need;
+    return EXAGO_OK;
+}
+
+void host_ranges(const BlockSym &S, DevSym &D) {
     D.k.nb = S.nb;
     D.k.nlevels = D.nlevels = S.nlevels;
     D.k.nblk = S.nblk;
@@ -766,6 +786,11 @@ int upload_block_sym(const BlockSym &S, DevSym &D, std::vector<void *> &allocs) 
     D.sparse_blocks = S.colptr[S.k0];
     D.k.k0 = S.k0;
     D.k.tail_n = S.tail_n;
+}
+
+int upload_block_sym(const BlockSym &S, DevSym &D, std::vector<void *> &allocs) {
+    D = DevSym();
+    host_ranges(S, D);
     auto up = [&](const void *src, size_t bytes, const void **dst) -> int {
         *dst = nullptr;
         if (bytes == 0) return 0;

@@ -29,6 +29,8 @@
 #include <string>
 #include <vector>
 
+#include "../../include/exago.h"
+
 namespace exago {
 
 struct BlockSym {
@@ -106,8 +108,14 @@ struct DevSym {
     int64_t sparse_blocks = 0;   // factor blocks of the columns before the tail
 };
 
+// D's host side: the launch ranges and the tail that S has by now (none before choose_tail).
+void host_ranges(const BlockSym &S, DevSym &D);
 // Uploads S (cudaMalloc through dev_malloc; the pointers go to `allocs` for the owner to free).
 int upload_block_sym(const BlockSym &S, DevSym &D, std::vector<void *> &allocs);
+
+// Grows a handle's internal workspace to `need` bytes; to `least`, enough without a dense tail, where the
+// device has no room for more.  What it then holds is in *bytes.
+exago_status grow_workspace(void **ws, size_t *bytes, size_t need, size_t least, const char *what);
 
 // Batched numeric factorisation and solve on DevSym.  T: the assembled matrix A, the lower blocks
 // of its own pattern (own_blk; and TU the upper blocks, the transposed positions, for LU),

@@ -246,7 +246,7 @@ struct exago_kkt {
     int device = -1;
     bool on_device = false;
     BlockSym S;
-    DevSym D;
+    DevSym D, all;            // with the dense tail; all columns level by level, for small workspaces
     KktDev K{};
     const int *own_blk = nullptr;   // device copy of S.own_blk
     std::vector<void *> allocs;
@@ -257,11 +257,11 @@ struct exago_kkt {
 
 namespace {
 
-size_t kkt_ws_bytes(const exago_kkt *k, int B) {
+size_t kkt_ws_bytes(const exago_kkt *k, const DevSym &D, int B) {
     const size_t entry = 16 * (size_t)B * sizeof(double);
-    return round256((size_t)k->S.nblk * entry) + round256((size_t)k->D.sparse_blocks * entry) +
+    return round256((size_t)k->S.nblk * entry) + round256((size_t)D.sparse_blocks * entry) +
            round256((size_t)k->S.nb * 4 * B * sizeof(double)) + round256(2 * (size_t)B * sizeof(int)) +
-           tail_shape(k->S.tail_n, B, true).bytes;
+           tail_shape(D.k.tail_n, B, true).bytes;
 }
 
 template <typename T>
@@ -329,8 +329,10 @@ exago_status exago_kkt_create(exago_net_t net, exago_kkt_t *out) {
             delete k;
             return set_last_error(EXAGO_EINVAL, "KKT symbolic factorisation: " + err);
         }
+        DevSym all;
+        host_ranges(k->S, all);
         choose_tail(k->S, 4, true);
-        k->D.sparse_blocks = k->S.colptr[k->S.k0];
+        host_ranges(k->S, k->D);
         const BlockSym &S = k->S;
         // variable / row index of entry a (0..3) of bus u: Va, Vm (x) or lamP, lamQ (rows)
         auto var = [&](int u, int a) { return a == 0 ? u : a == 1 ? nb + u : a == 2 ? u : nb + u; };
@@ -400,6 +402,10 @@ exago_status exago_kkt_create(exago_net_t net, exago_kkt_t *out) {
         exago_status s = EXAGO_OK;
         if (upload_block_sym(k->S, k->D, k->allocs) != 0) s = set_last_error(EXAGO_ENOMEM, "KKT symbolic tables");
         k->D.k.status = dev->status;   // the net's status word (debug-build index checks)
+        all.k = k->D.k;
+        all.k.k0 = nb;
+        all.k.tail_n = 0;
+        k->all = all;
         KktDev &K = k->K;
         K.nb = nb; K.nl = nl; K.ng = ng; K.n = n; K.m = m;
         K.nnzJ = P->nnzJ; K.nnzH = P->nnzH; K.nnzJg = P->nnzJg; K.hpg = P->Hrowptr[2 * nb];
@@ -466,7 +472,7 @@ exago_status exago_kkt_order(exago_kkt_t kkt, int *perm, int *parent, int *level
 exago_status exago_kkt_workspace_size(exago_kkt_t kkt, int B, size_t *bytes) {
     if (!kkt || !bytes) return set_last_error(EXAGO_EINVAL, "null argument");
     if (B < 0) return set_last_error(EXAGO_EINVAL, "B < 0");
-    *bytes = B == 0 ? 0 : kkt_ws_bytes(kkt, B);
+    *bytes = B == 0 ? 0 : kkt_ws_bytes(kkt, kkt->D, B);
     return EXAGO_OK;
 }
 
@@ -480,37 +486,28 @@ exago_status exago_kkt_solve(exago_kkt_t kkt, int B, const double *jval, const d
     if (B > 65535 * KNT) return set_last_error(EXAGO_EINVAL, "B too large for one call");
     if (!jval || !hval || !dx || !dc || !rhs || !sol)
         return set_last_error(EXAGO_EINVAL, "null input or output");
-    const size_t need = kkt_ws_bytes(kkt, B);
+    // Scratch for the dense tail, or at least for the factor's blocks: then no tail.
+    const size_t need = kkt_ws_bytes(kkt, kkt->D, B);
+    const size_t least = std::min(need, kkt_ws_bytes(kkt, kkt->all, B));
+    size_t have = workspace_bytes;
     cudaStream_t st = (cudaStream_t)stream;
     std::unique_lock<std::mutex> lk(kkt->mu, std::defer_lock);
     char *w = (char *)workspace;
     if (w) {
         if (((uintptr_t)w & 255) != 0) return set_last_error(EXAGO_EINVAL, "workspace not 256-byte aligned");
-        if (workspace_bytes < need) return set_last_error(EXAGO_EINVAL, "workspace smaller than exago_kkt_workspace_size");
+        if (have < least) return set_last_error(EXAGO_EINVAL, "workspace smaller than exago_kkt_workspace_size");
     } else {
         lk.lock();
-        if (kkt->ws_bytes < need) {
-            if (kkt->ws) {
-                cudaError_t e = cudaDeviceSynchronize();
-                if (e != cudaSuccess) return set_last_error(EXAGO_ECUDA, cudaGetErrorString(e));
-                cudaFree(kkt->ws);
-                kkt->ws = nullptr;
-                kkt->ws_bytes = 0;
-            }
-            cudaError_t e = dev_malloc(&kkt->ws, need);
-            if (e != cudaSuccess) {
-                kkt->ws = nullptr;
-                return set_last_error(e == cudaErrorMemoryAllocation ? EXAGO_ENOMEM : EXAGO_ECUDA,
-                                      "KKT workspace");
-            }
-            kkt->ws_bytes = need;
-        }
+        const exago_status s = grow_workspace(&kkt->ws, &kkt->ws_bytes, need, least, "KKT workspace");
+        if (s != EXAGO_OK) return s;
         w = (char *)kkt->ws;
+        have = kkt->ws_bytes;
     }
+    const DevSym &D = have >= need ? kkt->D : kkt->all;
     const size_t blk = round256((size_t)kkt->S.nblk * 16 * (size_t)B * sizeof(double));
     double *T = (double *)w;
     double *L = (double *)(w + blk);
-    char *p = w + blk + round256((size_t)kkt->D.sparse_blocks * 16 * (size_t)B * sizeof(double));
+    char *p = w + blk + round256((size_t)D.sparse_blocks * 16 * (size_t)B * sizeof(double));
     double *x = (double *)p;
     p += round256((size_t)kkt->S.nb * 4 * B * sizeof(double));
     int *neg = (int *)p, *bad = neg + B;
@@ -520,10 +517,10 @@ exago_status exago_kkt_solve(exago_kkt_t kkt, int B, const double *jval, const d
     cudaError_t e = cudaMemsetAsync(neg, 0, 2 * (size_t)B * sizeof(int), st);
     if (e != cudaSuccess) return set_last_error(EXAGO_ECUDA, cudaGetErrorString(e));
     k_kkt_assemble<<<dim3((unsigned)kkt->S.own_blk.size(), gy), KNT, 0, st>>>(
-        K, kkt->D.k, B, kkt->own_blk, jval, hval, dx, dc, T);
+        K, D.k, B, kkt->own_blk, jval, hval, dx, dc, T);
     k_kkt_rhs<<<dim3((unsigned)K.nb, gy), KNT, 0, st>>>(K, B, jval, hval, dx, dc, rhs, x, neg);
-    int le = launch_block_factor<4, true>(kkt->D, B, T, nullptr, L, nullptr, neg, bad, kTiny, tail, st);
-    if (le == 0) le = launch_block_solve<4, true>(kkt->D, B, T, L, nullptr, x, tail, st);
+    int le = launch_block_factor<4, true>(D, B, T, nullptr, L, nullptr, neg, bad, kTiny, tail, st);
+    if (le == 0) le = launch_block_solve<4, true>(D, B, T, L, nullptr, x, tail, st);
     if (le == 0) {
         k_kkt_recover_bus<<<dim3((unsigned)K.nb, gy), KNT, 0, st>>>(K, B, jval, hval, dx, rhs, x, sol);
         if (K.nl > 0)

@@ -105,7 +105,7 @@ struct exago_pf {
     const int *own_blk = nullptr;   // device copy of S.own_blk
     exago_net_t net = nullptr;
     BlockSym S;
-    DevSym D;
+    DevSym D, all;   // with the dense tail; all columns level by level, for small workspaces
     PfDev P{};
     std::vector<void *> allocs;
     std::mutex mu;
@@ -119,16 +119,16 @@ struct PfLayout {
     size_t gh, jv, blk, sblk, x, cnt, total;   // sblk: the columns before the dense tail
 };
 
-PfLayout pf_layout(const exago_pf *pf, int B) {
+PfLayout pf_layout(const exago_pf *pf, const DevSym &D, int B) {
     PfLayout L;
     L.gh = r256((size_t)B * pf->P.m * sizeof(double));
     L.jv = r256((size_t)B * pf->P.nnzJ * sizeof(double));
     L.blk = r256((size_t)pf->S.nblk * 4 * B * sizeof(double));
-    L.sblk = r256((size_t)pf->D.sparse_blocks * 4 * B * sizeof(double));
+    L.sblk = r256((size_t)D.sparse_blocks * 4 * B * sizeof(double));
     L.x = r256((size_t)pf->S.nb * 2 * B * sizeof(double));
     L.cnt = r256((size_t)B * (2 * sizeof(int) + sizeof(unsigned long long)));
     L.total = L.gh + L.jv + 2 * L.blk + 2 * L.sblk + L.x + L.cnt +
-              tail_shape(pf->S.tail_n, B, false).bytes;
+              tail_shape(D.k.tail_n, B, false).bytes;
     return L;
 }
 
@@ -202,6 +202,8 @@ exago_status exago_pf_create(exago_net_t net, const int *bus_type, exago_pf_t *o
             delete pf;
             return set_last_error(EXAGO_EINVAL, "power-flow symbolic factorisation: " + err);
         }
+        DevSym all;
+        host_ranges(pf->S, all);
         choose_tail(pf->S, 2, false);
         const BlockSym &S = pf->S;
         auto row_active = [&](int u, int a) { return a == 0 ? bus_type[u] != 3 : bus_type[u] == 1; };
@@ -228,6 +230,10 @@ exago_status exago_pf_create(exago_net_t net, const int *bus_type, exago_pf_t *o
         exago_status s = EXAGO_OK;
         if (upload_block_sym(pf->S, pf->D, pf->allocs) != 0) s = set_last_error(EXAGO_ENOMEM, "power-flow symbolic tables");
         pf->D.k.status = dev->status;   // the net's status word (debug-build index checks)
+        all.k = pf->D.k;
+        all.k.k0 = nb;
+        all.k.tail_n = 0;
+        pf->all = all;
         PfDev &D = pf->P;
         D.nb = nb; D.n = P->n; D.m = P->m; D.nnzJ = P->nnzJ;
         if (P->nnzJ >= (1ll << 31)) s = set_last_error(EXAGO_EINVAL, "grid too large");
@@ -260,7 +266,7 @@ exago_status exago_pf_destroy(exago_pf_t pf) {
 exago_status exago_pf_workspace_size(exago_pf_t pf, int B, size_t *bytes) {
     if (!pf || !bytes) return set_last_error(EXAGO_EINVAL, "null argument");
     if (B < 0) return set_last_error(EXAGO_EINVAL, "B < 0");
-    *bytes = B == 0 ? 0 : pf_layout(pf, B).total;
+    *bytes = B == 0 ? 0 : pf_layout(pf, pf->D, B).total;
     return EXAGO_OK;
 }
 
@@ -272,34 +278,26 @@ exago_status exago_pf_step(exago_pf_t pf, const exago_batch *batch, double *x_ne
     if (B == 0) return EXAGO_OK;
     if (B > 65535 * PNT) return set_last_error(EXAGO_EINVAL, "B too large for one call");
     if (!batch->x || !x_new) return set_last_error(EXAGO_EINVAL, "x or x_new is NULL");
-    const PfLayout Lw = pf_layout(pf, B);
+    // Scratch for the dense tail, or at least for the factor's blocks: then no tail.
+    const size_t need = pf_layout(pf, pf->D, B).total;
+    const size_t least = std::min(need, pf_layout(pf, pf->all, B).total);
+    size_t have = batch->workspace_bytes;
     cudaStream_t st = (cudaStream_t)batch->stream;
     std::unique_lock<std::mutex> lk(pf->mu, std::defer_lock);
     char *w = (char *)batch->workspace;
     if (w) {
         if (((uintptr_t)w & 255) != 0) return set_last_error(EXAGO_EINVAL, "workspace not 256-byte aligned");
-        if (batch->workspace_bytes < Lw.total)
+        if (have < least)
             return set_last_error(EXAGO_EINVAL, "workspace smaller than exago_pf_workspace_size");
     } else {
         lk.lock();
-        if (pf->ws_bytes < Lw.total) {
-            if (pf->ws) {
-                cudaError_t e = cudaDeviceSynchronize();
-                if (e != cudaSuccess) return set_last_error(EXAGO_ECUDA, cudaGetErrorString(e));
-                cudaFree(pf->ws);
-                pf->ws = nullptr;
-                pf->ws_bytes = 0;
-            }
-            cudaError_t e = dev_malloc(&pf->ws, Lw.total);
-            if (e != cudaSuccess) {
-                pf->ws = nullptr;
-                return set_last_error(e == cudaErrorMemoryAllocation ? EXAGO_ENOMEM : EXAGO_ECUDA,
-                                      "power-flow workspace");
-            }
-            pf->ws_bytes = Lw.total;
-        }
+        const exago_status s = grow_workspace(&pf->ws, &pf->ws_bytes, need, least, "power-flow workspace");
+        if (s != EXAGO_OK) return s;
         w = (char *)pf->ws;
+        have = pf->ws_bytes;
     }
+    const DevSym &Ds = have >= need ? pf->D : pf->all;
+    const PfLayout Lw = pf_layout(pf, Ds, B);
     double *gh = (double *)w;
     double *jv = (double *)(w + Lw.gh);
     char *fw = w + Lw.gh + Lw.jv;
@@ -325,8 +323,8 @@ exago_status exago_pf_step(exago_pf_t pf, const exago_batch *batch, double *x_ne
     const unsigned gy = (unsigned)((B + PNT - 1) / PNT);
     k_pf_assemble<<<dim3((unsigned)pf->S.own_blk.size(), gy), PNT, 0, st>>>(D, B, pf->own_blk, jv, T, TU);
     k_pf_rhs<<<dim3((unsigned)D.nb, gy), PNT, 0, st>>>(D, B, gh, x, mis);
-    int le = launch_block_factor<2, false>(pf->D, B, T, TU, L, U, neg, bad, kPfTiny, tail, st);
-    if (le == 0) le = launch_block_solve<2, false>(pf->D, B, T, L, U, x, tail, st);
+    int le = launch_block_factor<2, false>(Ds, B, T, TU, L, U, neg, bad, kPfTiny, tail, st);
+    if (le == 0) le = launch_block_solve<2, false>(Ds, B, T, L, U, x, tail, st);
     if (le == 0) {
         k_pf_update<<<dim3((unsigned)D.n, gy), PNT, 0, st>>>(D, B, batch->x, x, x_new);
         if (mismatch) k_pf_mismatch<<<(B + 255) / 256, 256, 0, st>>>(mis, mismatch, B);
