@@ -65,6 +65,7 @@ struct BlockSym {
     // pairs with K < k0; tail_r1 [nb]: end of each row's blocks with K < k0; tail_tgt: the target
     // of each lower block (I, J) of the tail, row after row, or -1 where the factor has none.
     int k0 = 0, tail_n = 0;          // first tail column; padded scalar size
+    int tail_most = 0;               // the largest batch that the tail is taken for (tail_most_states)
     // sp_pairs, sp_rows, sp_colblks [nlevels]: the most pairs of a target, blocks (J, K) of a row and
     // blocks (I, J) of a column among the level's columns below k0.
     std::vector<int> sp_cols, sp_tgts, sp_pairs, sp_rows, sp_colblks, tail_tgt;
@@ -78,8 +79,9 @@ struct BlockSym {
 // inconsistent graph.
 bool build_block_sym(int nb, const int *adj_ptr, const int *adj, BlockSym &S, std::string &err);
 
-// Chooses the dense tail of a factorisation of BS x BS blocks (symmetric or not) from the structure
-// alone, so that a state's factorisation is the same in every batch.
+// Chooses the dense tail of a factorisation of BS x BS blocks (symmetric or not), and the largest
+// batch that it is taken for, from the structure alone: a state's factorisation is the same in every
+// batch up to that size, and in every larger one.
 void choose_tail(BlockSym &S, int BS, bool sym);
 
 // Device tables of a symbolic factorisation (handed to the kernels by value).

@@ -7,6 +7,7 @@
 // are enough.  Plain host code (no CUDA calls): the host tests build it with the address and
 // undefined-behaviour sanitizers.
 #include <algorithm>
+#include <climits>
 #include <cstdio>
 #include <set>
 
@@ -47,6 +48,31 @@ void sparse_levels(BlockSym &S) {
         for (int t = S.lvl_tptr[l]; t < S.lvl_tptr[l] + S.sp_tgts[l]; t++)
             S.sp_pairs[l] = std::max(S.sp_pairs[l], (int)(S.tptr[t + 1] - S.tptr[t]));
     }
+}
+
+// The largest batch for which the tail is faster than the same columns level by level.  The tail saves
+// launches and the chains of narrow levels, but a 64-column panel costs its 64 dense pivots however
+// few of its blocks the factor has, so small grids in large batches are faster without it.  Fitted to 39
+// grids of 3 to 300 buses and 1.35 to 3 branches a bus x 1 to 16,384 states, both ways (us, c the
+// columns of the tail): level by level per state 1.15e-4 a block product + 4.9e-4 a block, and 34
+// a level + 0.028 a product + 0.46 a block with 128 states; panels per state 0.33 each + 0.104 a tile
+// product, and 150 each with 128 states, up to which an SM has one block (2 x 2 blocks, LU: the second
+// set).  The choice is at most 7% off the better one on any of them.  Without the line (tail, level by level):
+// KKT 14 buses x 4,096 1,463 and 303 us, 57 x 16,384 6,899 and 2,803, 118 x 512 634 and 906; power
+// flow 57 buses x 2,048 1,369 and 413, 300 x 512 737 and 1,141.
+int tail_most_states(const BlockSym &S, int BS, double products) {
+    const double P = S.tail_n / 64, tiles = P * (P + 1) * (P + 2) / 6 - P;
+    int levels = 0;
+    for (int k = 0; k < S.k0; k++) levels = std::max(levels, S.level[k] + 1);
+    levels = S.nlevels - levels;
+    const double blocks = (double)(S.nblk - S.colptr[S.k0]);
+    const bool kkt = BS == 4;
+    const double state = kkt ? 1.15e-4 * products + 4.9e-4 * blocks - 0.33 * P - 0.104 * tiles
+                             : 2.9e-5 * products + 1.4e-4 * blocks - 0.55 * P - 0.19 * tiles;
+    const double fixed = kkt ? 34.0 * levels + 0.028 * products + 0.46 * blocks - 150.0 * P
+                             : 21.0 * levels + 0.008 * products + 0.11 * blocks - 160.0 * P;
+    if (fixed < 0) return state < 0 ? 0 : INT_MAX;
+    return state < 0 ? (int)std::min(1e9, 128.0 + fixed / -state) : INT_MAX;
 }
 
 }  // namespace
@@ -242,6 +268,12 @@ void choose_tail(BlockSym &S, int BS, bool sym) {
     const int k0 = best_k0, R = nb - k0;
     S.k0 = k0;
     S.tail_n = best_n;
+    S.tail_most = tail_most_states(S, BS, pairs[nb] - pairs[k0]);
+    if (S.tail_most == 0) {
+        S.k0 = nb;
+        S.tail_n = 0;
+        return;
+    }
     sparse_levels(S);
     std::vector<int> col_of_blk(S.nblk);
     for (int k = 0; k < nb; k++)

@@ -472,7 +472,9 @@ exago_status exago_kkt_order(exago_kkt_t kkt, int *perm, int *parent, int *level
 exago_status exago_kkt_workspace_size(exago_kkt_t kkt, int B, size_t *bytes) {
     if (!kkt || !bytes) return set_last_error(EXAGO_EINVAL, "null argument");
     if (B < 0) return set_last_error(EXAGO_EINVAL, "B < 0");
-    *bytes = B == 0 ? 0 : kkt_ws_bytes(kkt, kkt->D, B);
+    // enough for every smaller batch too
+    *bytes = B == 0 ? 0 : kkt_ws_bytes(kkt, kkt->D, std::min(B, kkt->S.tail_most));
+    if (B > kkt->S.tail_most) *bytes = std::max(*bytes, kkt_ws_bytes(kkt, kkt->all, B));
     return EXAGO_OK;
 }
 
@@ -487,8 +489,9 @@ exago_status exago_kkt_solve(exago_kkt_t kkt, int B, const double *jval, const d
     if (!jval || !hval || !dx || !dc || !rhs || !sol)
         return set_last_error(EXAGO_EINVAL, "null input or output");
     // Scratch for the dense tail, or at least for the factor's blocks: then no tail.
-    const size_t need = kkt_ws_bytes(kkt, kkt->D, B);
-    const size_t least = std::min(need, kkt_ws_bytes(kkt, kkt->all, B));
+    const size_t tail_need = kkt_ws_bytes(kkt, kkt->D, B), all_need = kkt_ws_bytes(kkt, kkt->all, B);
+    const bool want_tail = B <= kkt->S.tail_most;
+    const size_t need = want_tail ? tail_need : all_need, least = std::min(need, all_need);
     size_t have = workspace_bytes;
     cudaStream_t st = (cudaStream_t)stream;
     std::unique_lock<std::mutex> lk(kkt->mu, std::defer_lock);
@@ -503,7 +506,7 @@ exago_status exago_kkt_solve(exago_kkt_t kkt, int B, const double *jval, const d
         w = (char *)kkt->ws;
         have = kkt->ws_bytes;
     }
-    const DevSym &D = have >= need ? kkt->D : kkt->all;
+    const DevSym &D = want_tail && have >= need ? kkt->D : kkt->all;
     const size_t blk = round256((size_t)kkt->S.nblk * 16 * (size_t)B * sizeof(double));
     double *T = (double *)w;
     double *L = (double *)(w + blk);

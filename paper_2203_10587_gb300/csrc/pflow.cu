@@ -266,7 +266,9 @@ exago_status exago_pf_destroy(exago_pf_t pf) {
 exago_status exago_pf_workspace_size(exago_pf_t pf, int B, size_t *bytes) {
     if (!pf || !bytes) return set_last_error(EXAGO_EINVAL, "null argument");
     if (B < 0) return set_last_error(EXAGO_EINVAL, "B < 0");
-    *bytes = B == 0 ? 0 : pf_layout(pf, pf->D, B).total;
+    // enough for every smaller batch too
+    *bytes = B == 0 ? 0 : pf_layout(pf, pf->D, std::min(B, pf->S.tail_most)).total;
+    if (B > pf->S.tail_most) *bytes = std::max(*bytes, pf_layout(pf, pf->all, B).total);
     return EXAGO_OK;
 }
 
@@ -279,8 +281,9 @@ exago_status exago_pf_step(exago_pf_t pf, const exago_batch *batch, double *x_ne
     if (B > 65535 * PNT) return set_last_error(EXAGO_EINVAL, "B too large for one call");
     if (!batch->x || !x_new) return set_last_error(EXAGO_EINVAL, "x or x_new is NULL");
     // Scratch for the dense tail, or at least for the factor's blocks: then no tail.
-    const size_t need = pf_layout(pf, pf->D, B).total;
-    const size_t least = std::min(need, pf_layout(pf, pf->all, B).total);
+    const size_t tail_need = pf_layout(pf, pf->D, B).total, all_need = pf_layout(pf, pf->all, B).total;
+    const bool want_tail = B <= pf->S.tail_most;
+    const size_t need = want_tail ? tail_need : all_need, least = std::min(need, all_need);
     size_t have = batch->workspace_bytes;
     cudaStream_t st = (cudaStream_t)batch->stream;
     std::unique_lock<std::mutex> lk(pf->mu, std::defer_lock);
@@ -296,7 +299,7 @@ exago_status exago_pf_step(exago_pf_t pf, const exago_batch *batch, double *x_ne
         w = (char *)pf->ws;
         have = pf->ws_bytes;
     }
-    const DevSym &Ds = have >= need ? pf->D : pf->all;
+    const DevSym &Ds = want_tail && have >= need ? pf->D : pf->all;
     const PfLayout Lw = pf_layout(pf, Ds, B);
     double *gh = (double *)w;
     double *jv = (double *)(w + Lw.gh);

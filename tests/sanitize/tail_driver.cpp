@@ -1,6 +1,6 @@
 // Test driver: reads "buses branches" and the branches' end buses, prints the dense tail that the
 // block factorisation chooses for it (choose_tail): first tail column and padded scalar size of the
-// KKT step (4 x 4 blocks) and of the power-flow step (2 x 2).  Built by tests/test_tail_shapes.py.
+// KKT step (4 x 4 blocks) and of the power-flow step (2 x 2), and the largest batch it is taken for.  Built by tests/test_tail_shapes.py.
 #include <cstdio>
 #include <string>
 #include <vector>
@@ -22,7 +22,7 @@ int main() {
         std::string err;
         if (!exago::build_block_sym(nb, ptr.data(), adj.data(), S, err)) return 2;
         exago::choose_tail(S, bs, bs == 4);
-        printf("%d %d\n", S.k0, S.tail_n);
+        printf("%d %d %d\n", S.k0, S.tail_n, S.tail_most);
     }
     return 0;
 }
