@@ -9,10 +9,10 @@
 // constants +1 / -1, and they add nothing to the Lagrangian Hessian.  The transpose product is a
 // gather over each state's children, in a fixed order (no atomics):
 //     (C^T nu)[b][Pg_k] = [p(b) >= 0] nu[b][k] - sum over children c of b of nu[c][k].
-// States with few children are summed by one thread per (state, generator); a state with many
-// children (the base case of a contingency or scenario batch) is summed by blocks of 4 generators
-// whose 64 rows of threads take every 64th child of the list staged in shared memory and then
-// reduce in a fixed tree.
+// States with few children are summed by one thread per (state, generator); a state with more than 256
+// (the base case of a contingency or scenario batch) by blocks of 4 generators whose 64 rows of threads
+// take every 64th child of the list staged in shared memory and then reduce in a fixed tree, one with 9 to 256
+// by blocks of 8 generators and 32 rows.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,9 +26,9 @@ struct exago_coupling {
     int B = 0, nb = 0, ng = 0, n = 0;
     bool on_device = false;
     int device = -1;
-    std::vector<int> parent, child_ptr, child_idx, light, heavy;
+    std::vector<int> parent, child_ptr, child_idx, light, some, many;   // states by number of children
     int *d_parent = nullptr, *d_child_ptr = nullptr, *d_child_idx = nullptr;
-    int *d_light = nullptr, *d_heavy = nullptr;
+    int *d_light = nullptr, *d_some = nullptr, *d_many = nullptr;
     void *d_mem = nullptr;
 };
 
@@ -36,9 +36,10 @@ namespace {
 
 using exago::set_last_error;
 
-// A state with more children than this is reduced by blocks of kHeavyCols x kHeavyRows.
-constexpr int kHeavyChildren = 8;
-constexpr int kHeavyCols = 4, kHeavyRows = 64;   // generators x child lanes of such a block
+// A state with more children than these is reduced by blocks of kSomeCols or kManyCols generators and
+// 256 / that rows of threads for its children (8 batched loads a thread cover 256 children with 32 rows).
+constexpr int kSomeChildren = 8, kManyChildren = 256;
+constexpr int kSomeCols = 8, kManyCols = 4;
 constexpr int kMaxGridY = 65535;
 // Children of a heavy state staged in shared memory per pass.
 constexpr int kStageChildren = 2048;
@@ -77,54 +78,64 @@ __device__ __forceinline__ void put(double *o, double v, int accumulate) {
 }
 
 struct JtvArgs {
-    const int *light, *heavy, *parent, *cptr, *cidx;
-    int nheavy, hblocks, lblocks, ng, accumulate;   // hblocks, lblocks: blocks of one state
+    const int *light, *some, *many, *parent, *cptr, *cidx;
+    int nsome, nmany, sblocks, mblocks, lblocks, ng, accumulate;   // .blocks: blocks of one state
     const double *nu;
     double *out;
     int64_t ldo;
 };
 
-// One launch for all states (256 threads a block): first the heavy ones, hblocks blocks of
-// kHeavyCols generators each, then the light ones, lblocks blocks of kRowSpan generators each.
-//   * heavy: the state's children are staged in shared memory, thread row ty sums children ty,
-//     ty + kHeavyRows, ... (independent loads), and the partial sums are reduced by a fixed halving
-//     tree.  A 512-state star: 8 children a thread in one batch of loads; with 8 generators x 32
-//     rows they were two, in a launch of its own (15.6 us the two launches);
-//   * light: the state's own row minus its children's, in ascending order.
-__global__ void __launch_bounds__(256) k_coupling_jtv(const JtvArgs A) {
-    __shared__ int kids[kStageChildren];
-    __shared__ double part[kHeavyRows][kHeavyCols + 1];
-    const int tid = threadIdx.x, ng = A.ng;
-    const int64_t heavy_blocks = (int64_t)A.nheavy * A.hblocks;
-    if ((int64_t)blockIdx.x < heavy_blocks) {
-        const int tx = tid % kHeavyCols, ty = tid / kHeavyCols;
-        const int s = __ldg(A.heavy + blockIdx.x / A.hblocks);
-        const int k = (blockIdx.x % A.hblocks) * kHeavyCols + tx;
-        const int c0 = __ldg(A.cptr + s), c1 = __ldg(A.cptr + s + 1);
-        double acc = 0.0;
-        for (int base = c0; base < c1; base += kStageChildren) {
-            const int cnt = min(kStageChildren, c1 - base);
-            __syncthreads();   // the previous pass is done with kids
-            for (int j = tid; j < cnt; j += 256) kids[j] = __ldg(A.cidx + base + j);
-            __syncthreads();
-            if (k < ng) {
-#pragma unroll 8
-                for (int j = ty; j < cnt; j += kHeavyRows) acc += __ldg(A.nu + (int64_t)kids[j] * ng + k);
-            }
-        }
-        part[ty][tx] = acc;
+// Block g of COLS generators of state s: its children are staged in shared memory, thread row ty sums
+// children ty, ty + ROWS, ... (independent loads), and the partial sums are reduced by a fixed halving tree.
+template <int COLS>
+__device__ __forceinline__ void sum_children(const JtvArgs &A, int s, int g, int *kids, double *part) {
+    constexpr int ROWS = 256 / COLS, PITCH = COLS + 1;
+    const int tid = threadIdx.x, tx = tid % COLS, ty = tid / COLS, ng = A.ng, k = g * COLS + tx;
+    const int c0 = __ldg(A.cptr + s), c1 = __ldg(A.cptr + s + 1);
+    double acc = 0.0;
+    for (int base = c0; base < c1; base += kStageChildren) {
+        const int cnt = min(kStageChildren, c1 - base);
+        __syncthreads();   // the previous pass is done with kids
+        for (int j = tid; j < cnt; j += 256) kids[j] = __ldg(A.cidx + base + j);
         __syncthreads();
-        for (int h = kHeavyRows / 2; h >= 1; h >>= 1) {
-            if (ty < h) part[ty][tx] += part[ty + h][tx];
-            __syncthreads();
+        if (k < ng) {
+#pragma unroll 8
+            for (int j = ty; j < cnt; j += ROWS) acc += __ldg(A.nu + (int64_t)kids[j] * ng + k);
         }
-        if (ty == 0 && k < ng) {
-            const double own = __ldg(A.parent + s) >= 0 ? __ldg(A.nu + (int64_t)s * ng + k) : 0.0;
-            put(A.out + (int64_t)s * A.ldo + k, own - part[0][tx], A.accumulate);
-        }
+    }
+    part[ty * PITCH + tx] = acc;
+    __syncthreads();
+    for (int h = ROWS / 2; h >= 1; h >>= 1) {
+        if (ty < h) part[ty * PITCH + tx] += part[(ty + h) * PITCH + tx];
+        __syncthreads();
+    }
+    if (ty == 0 && k < ng) {
+        const double own = __ldg(A.parent + s) >= 0 ? __ldg(A.nu + (int64_t)s * ng + k) : 0.0;
+        put(A.out + (int64_t)s * A.ldo + k, own - part[tx], A.accumulate);
+    }
+}
+
+// One launch for all states (256 threads a block): first those with many children, mblocks blocks of
+// kManyCols generators each, then those with some, sblocks blocks of kSomeCols, then the light ones,
+// lblocks blocks of kRowSpan generators each: the state's own row minus its children's, in ascending order.
+// A 512-state star (many): 8 children a thread in one batch of loads; with 8 generators x 32 rows they
+// were two, in a launch of its own (15.6 us the two launches).  With a dozen children a state the narrow
+// blocks are twice as many for nothing: 900 buses x 4,096 states 55 us with 4 generators a block, 30 with 8.
+__global__ void __launch_bounds__(256, 8) k_coupling_jtv(const JtvArgs A) {
+    __shared__ int kids[kStageChildren];
+    __shared__ double part[256 + 256 / kManyCols];
+    const int tid = threadIdx.x, ng = A.ng;
+    const unsigned many_blocks = A.nmany * A.mblocks, some_blocks = A.nsome * A.sblocks;   // a grid holds all
+    if (blockIdx.x < many_blocks) {
+        sum_children<kManyCols>(A, __ldg(A.many + blockIdx.x / A.mblocks), blockIdx.x % A.mblocks, kids, part);
         return;
     }
-    const int64_t blk = (int64_t)blockIdx.x - heavy_blocks;
+    if (blockIdx.x < many_blocks + some_blocks) {
+        const unsigned q = blockIdx.x - many_blocks;
+        sum_children<kSomeCols>(A, __ldg(A.some + q / A.sblocks), q % A.sblocks, kids, part);
+        return;
+    }
+    const unsigned blk = blockIdx.x - many_blocks - some_blocks;
     const int s = __ldg(A.light + blk / A.lblocks);
     const bool own = __ldg(A.parent + s) >= 0;
     const int c0 = __ldg(A.cptr + s), c1 = __ldg(A.cptr + s + 1);
@@ -152,7 +163,6 @@ __global__ void __launch_bounds__(256) k_coupling_jtv(const JtvArgs A) {
     }
 }
 
-// Blocks along a row of ng values: one 256-thread block per kRowSpan values.
 exago_status check_call(exago_coupling_t c) {
     if (!c) return set_last_error(EXAGO_EINVAL, "coupling is NULL");
     if (!c->on_device)
@@ -207,8 +217,10 @@ exago_status exago_coupling_create(exago_net_t net, int B, const int *parent,
         for (int b = 0; b < B; b++)   // ascending child order
             if (parent[b] >= 0) c->child_idx[fill[parent[b]]++] = b;
     }
-    for (int b = 0; b < B; b++)
-        (c->child_ptr[b + 1] - c->child_ptr[b] > kHeavyChildren ? c->heavy : c->light).push_back(b);
+    for (int b = 0; b < B; b++) {
+        const int nc = c->child_ptr[b + 1] - c->child_ptr[b];
+        (nc > kManyChildren ? c->many : nc > kSomeChildren ? c->some : c->light).push_back(b);
+    }
 
     const exago::HostPlan *plan = nullptr;
     const exago::DevNet *dev = nullptr;
@@ -222,8 +234,8 @@ exago_status exago_coupling_create(exago_net_t net, int B, const int *parent,
                                   e != cudaSuccess ? cudaGetErrorString(e)
                                                    : "make the net's device current before the call");
         }
-        // one allocation: parent [B], child_ptr [B + 1], child_idx, light, heavy
-        const size_t ints = (size_t)B + (B + 1) + c->child_idx.size() + c->light.size() + c->heavy.size();
+        // one allocation: parent [B], child_ptr [B + 1], child_idx, light, some, many
+        const size_t ints = (size_t)B + (B + 1) + c->child_idx.size() + B;
         e = exago::dev_malloc(&c->d_mem, std::max<size_t>(ints, 1) * sizeof(int));
         if (e != cudaSuccess) {
             delete c;
@@ -235,7 +247,8 @@ exago_status exago_coupling_create(exago_net_t net, int B, const int *parent,
         all.insert(all.end(), c->child_ptr.begin(), c->child_ptr.end());
         all.insert(all.end(), c->child_idx.begin(), c->child_idx.end());
         all.insert(all.end(), c->light.begin(), c->light.end());
-        all.insert(all.end(), c->heavy.begin(), c->heavy.end());
+        all.insert(all.end(), c->some.begin(), c->some.end());
+        all.insert(all.end(), c->many.begin(), c->many.end());
         if (!all.empty()) {
             e = cudaMemcpy(c->d_mem, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice);
             if (e != cudaSuccess) {
@@ -254,7 +267,9 @@ exago_status exago_coupling_create(exago_net_t net, int B, const int *parent,
         p += c->child_idx.size();
         c->d_light = p;
         p += c->light.size();
-        c->d_heavy = p;
+        c->d_some = p;
+        p += c->some.size();
+        c->d_many = p;
     }
     *out = c;
     return EXAGO_OK;
@@ -328,16 +343,19 @@ exago_status exago_eval_coupling_jtv(exago_coupling_t c, const double *nu, doubl
     if (!nu || !out) return set_last_error(EXAGO_EINVAL, "nu or out is NULL");
     if (ldo < c->ng) return set_last_error(EXAGO_EINVAL, "ldo < ng");
     cudaStream_t s = (cudaStream_t)stream;
-    const int nlight = (int)c->light.size(), nheavy = (int)c->heavy.size();
+    const int nlight = (int)c->light.size(), nsome = (int)c->some.size(), nmany = (int)c->many.size();
     // states of one launch, so that its blocks fit the grid (2^31 - 1)
-    const int hb = (c->ng + kHeavyCols - 1) / kHeavyCols, lb = (int)row_blocks(c->ng);
-    const int hmax = std::max(1, (1 << 30) / hb), lmax = std::max(1, (1 << 30) / lb);
-    for (int h0 = 0, l0 = 0; h0 < nheavy || l0 < nlight;) {
-        const int nh = std::min(hmax, nheavy - h0), nl = std::min(lmax, nlight - l0);
-        const JtvArgs A{c->d_light + l0, c->d_heavy + h0, c->d_parent, c->d_child_ptr, c->d_child_idx,
-                        nh, hb, lb, c->ng, accumulate ? 1 : 0, nu, out, ldo};
-        k_coupling_jtv<<<(unsigned)(nh * hb + nl * lb), 256, 0, s>>>(A);
-        h0 += nh;
+    const int mb = (c->ng + kManyCols - 1) / kManyCols, sb = (c->ng + kSomeCols - 1) / kSomeCols;
+    const int lb = (int)row_blocks(c->ng);
+    auto most = [](int blocks) { return std::max(1, (1 << 29) / blocks); };
+    for (int m0 = 0, s0 = 0, l0 = 0; m0 < nmany || s0 < nsome || l0 < nlight;) {
+        const int nm = std::min(most(mb), nmany - m0), ns = std::min(most(sb), nsome - s0);
+        const int nl = std::min(most(lb), nlight - l0);
+        const JtvArgs A{c->d_light + l0, c->d_some + s0, c->d_many + m0, c->d_parent, c->d_child_ptr,
+                        c->d_child_idx, ns, nm, sb, mb, lb, c->ng, accumulate ? 1 : 0, nu, out, ldo};
+        k_coupling_jtv<<<(unsigned)(nm * mb + ns * sb + nl * lb), 256, 0, s>>>(A);
+        m0 += nm;
+        s0 += ns;
         l0 += nl;
     }
     cudaError_t e = cudaGetLastError();
