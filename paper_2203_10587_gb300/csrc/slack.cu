@@ -66,19 +66,23 @@ struct SlackArgs {
     int64_t ldgh;
 };
 
-// For the states b0 + kStates y ..: blocks x < kStates do the objective of one state each, then
-// row_blocks blocks the rows and grad_blocks the gradient of all of them.  One launch in place of
+// For the states b0 + kStates y ..: blocks x < kStates do the objective of one state each (OBJ), then
+// row_blocks blocks the rows (ROWS) and the rest the gradient (GRAD) of all of them; an instance for each
+// set of outputs, since blocks for absent ones and their registers cost a call of one output over
+// 16,384 small states a third of its time (14 buses, rows alone: 9.4 us, 14.7 with them).  One launch in place of
 // three, each of which waited for the one before.  Bound by the FP64 pipe (an addition a slack
 // for the rows and a multiply-add for the objective: 18 us on 2,000 buses x 512 states, 10,766
 // slacks a state), so the gradient's products go to the integer pipe.  69 us in three launches
 // with FP64 sign and gradient products, 41 now.
+template <bool OBJ, bool ROWS, bool GRAD>
 __global__ void __launch_bounds__(kLanes) k_slack_apply(const SlackArgs A) {
-    __shared__ double part[kLanes];
-    const int tid = threadIdx.x, bs = A.b0 + kStates * blockIdx.y, nz = A.nz;
-    const int ns = min(kStates, A.b0 + A.nB - bs);
+    __shared__ double part[OBJ ? kLanes : 1];
+    constexpr int S = OBJ || ROWS ? kStates : 1;   // the gradient alone has few blocks otherwise
+    const int tid = threadIdx.x, bs = A.b0 + S * blockIdx.y, nz = A.nz;
+    const int ns = min(S, A.b0 + A.nB - bs);
     int x = blockIdx.x;
-    if (x < kStates) {
-        if (!A.f || x >= ns) return;
+    if (OBJ && x < kStates) {
+        if (x >= ns) return;
         const int b = bs + x;
         const double *zb = A.z + (int64_t)b * nz;
         double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
@@ -99,8 +103,8 @@ __global__ void __launch_bounds__(kLanes) k_slack_apply(const SlackArgs A) {
         if (tid == 0) A.f[b] = fma(A.obj_weight ? __ldg(A.obj_weight + b) : 1.0, part[0], A.f[b]);
         return;
     }
-    x -= kStates;
-    if (x < A.row_blocks) {
+    if (OBJ) x -= kStates;
+    if (ROWS && x < A.row_blocks) {
         const int j = x * kLanes + tid;
         if (j >= A.nused) return;
         const int2 row = __ldg(A.rows + j);
@@ -129,7 +133,8 @@ __global__ void __launch_bounds__(kLanes) k_slack_apply(const SlackArgs A) {
             if (t < ns) g[t * A.ldgh] = v[t];
         return;
     }
-    x -= A.row_blocks;
+    if (!GRAD) return;
+    if (ROWS) x -= A.row_blocks;
 #pragma unroll
     for (int u = 0; u < kPart / kLanes; u++) {
         const int k = x * kPart + u * kLanes + tid;
@@ -137,27 +142,31 @@ __global__ void __launch_bounds__(kLanes) k_slack_apply(const SlackArgs A) {
         const double c = __ldg(A.cost + k);
         for (int t = 0; t < ns; t++) {
             const double w = A.obj_weight ? __ldg(A.obj_weight + bs + t) : 1.0;
-            A.grad_z[(int64_t)(bs + t) * nz + k] = mul_window(w) && mul_window(c) ? int_mul(w, c)
-                                                                                  : fp_mul(w, c);
+            // alone, the FP64 pipe is free for the products (integer ones take 1.25 times as long)
+            if (!OBJ && !ROWS) A.grad_z[(int64_t)(bs + t) * nz + k] = w * c;
+            else A.grad_z[(int64_t)(bs + t) * nz + k] = mul_window(w) && mul_window(c) ? int_mul(w, c)
+                                                                                       : fp_mul(w, c);
         }
     }
 }
 
-// out[b][k] = sign_k v[b][row_k]: every load of a thread's four slacks before its first store.
+// out[b][k] = sign_k v[b][row_k]: every load of a thread's U slacks before its first store (four, or one
+// where a state has no more slacks than a block has threads).
+template <int U>
 __global__ void __launch_bounds__(256) k_slack_jtv(const unsigned *__restrict__ gcode, int nz, int b0,
                                                    const double *__restrict__ v, int64_t ldv,
                                                    double *__restrict__ out) {
-    const int b = b0 + blockIdx.y, k0 = blockIdx.x * 1024 + threadIdx.x;
+    const int b = b0 + blockIdx.y, k0 = blockIdx.x * (256 * U) + threadIdx.x;
     const double *vb = v + (int64_t)b * ldv;
     double *ob = out + (int64_t)b * nz;
-    unsigned c[4];
-    double t[4];
+    unsigned c[U];
+    double t[U];
 #pragma unroll
-    for (int u = 0; u < 4; u++) c[u] = k0 + u * 256 < nz ? __ldg(gcode + k0 + u * 256) : 0;
+    for (int u = 0; u < U; u++) c[u] = k0 + u * 256 < nz ? __ldg(gcode + k0 + u * 256) : 0;
 #pragma unroll
-    for (int u = 0; u < 4; u++) t[u] = k0 + u * 256 < nz ? __ldg(vb + (c[u] >> 1)) : 0.0;
+    for (int u = 0; u < U; u++) t[u] = k0 + u * 256 < nz ? __ldg(vb + (c[u] >> 1)) : 0.0;
 #pragma unroll
-    for (int u = 0; u < 4; u++)
+    for (int u = 0; u < U; u++)
         if (k0 + u * 256 < nz) ob[k0 + u * 256] = signed_by(t[u], c[u]);
 }
 
@@ -298,8 +307,18 @@ exago_status exago_eval_slack(exago_slack_t s, const exago_batch *bt, const doub
             SlackArgs C = L;
             C.b0 = b0;
             C.nB = std::min(kMaxGridY, bt->B - b0);
-            k_slack_apply<<<dim3(kStates + C.row_blocks + C.grad_blocks, (C.nB + kStates - 1) / kStates),
-                            kLanes, 0, stream>>>(C);
+            const int S = C.f || C.gh ? kStates : 1;
+            const dim3 grid((C.f ? S : 0) + C.row_blocks + C.grad_blocks, (C.nB + S - 1) / S);
+            if (grid.x == 0) continue;   // rows alone, and none has a slack
+            switch ((C.f ? 1 : 0) | (C.gh ? 2 : 0) | (C.grad_z ? 4 : 0)) {
+                case 1: k_slack_apply<true, false, false><<<grid, kLanes, 0, stream>>>(C); break;
+                case 2: k_slack_apply<false, true, false><<<grid, kLanes, 0, stream>>>(C); break;
+                case 3: k_slack_apply<true, true, false><<<grid, kLanes, 0, stream>>>(C); break;
+                case 4: k_slack_apply<false, false, true><<<grid, kLanes, 0, stream>>>(C); break;
+                case 5: k_slack_apply<true, false, true><<<grid, kLanes, 0, stream>>>(C); break;
+                case 6: k_slack_apply<false, true, true><<<grid, kLanes, 0, stream>>>(C); break;
+                default: k_slack_apply<true, true, true><<<grid, kLanes, 0, stream>>>(C); break;
+            }
         }
     };
     const uintptr_t span = (uintptr_t)bt->B * s->nz * sizeof(double), dist = (uintptr_t)grad_z - (uintptr_t)z;
@@ -339,8 +358,10 @@ exago_status exago_eval_slack_jtv(exago_slack_t s, const exago_batch *bt, const 
     if (ldv < 2 * s->nb) return set_last_error(EXAGO_EINVAL, "ldv < 2 nb");
     for (int b0 = 0; b0 < bt->B; b0 += kMaxGridY) {
         const int nB = std::min(kMaxGridY, bt->B - b0);
-        k_slack_jtv<<<dim3((s->nz + 1023) / 1024, nB), 256, 0, (cudaStream_t)bt->stream>>>(
-            (const unsigned *)s->d_int + 2 * (s->used.size() + 1), s->nz, b0, v, ldv, out);
+        const unsigned *code = (const unsigned *)s->d_int + 2 * (s->used.size() + 1);
+        const cudaStream_t cs = (cudaStream_t)bt->stream;
+        if (s->nz <= 256) k_slack_jtv<1><<<dim3(1, nB), 256, 0, cs>>>(code, s->nz, b0, v, ldv, out);
+        else k_slack_jtv<4><<<dim3((s->nz + 1023) / 1024, nB), 256, 0, cs>>>(code, s->nz, b0, v, ldv, out);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
