@@ -570,7 +570,7 @@ def run_kkt(exago, synth, torch, np, dev, reps=10, warm=2):
     dc ~ U(0.5, 2), rhs ~ N(0, 1): assembly, eliminations, the batched block L D L' and both
     sweeps, CUDA events over back-to-back calls.  FP64-bound: the flops per state are
     exago_kkt_info's count (its 4 x 4 block products dominate).  Most of those products run on the
-    tensor cores, exactly split, so frac_fp64_peak may exceed 1."""
+    tensor cores, in 62-bit fixed point, so frac_fp64_peak may exceed 1."""
     g = synth.grid_2000()
     b = synth.contingency_batch(3, g, 512)
     B = b.B

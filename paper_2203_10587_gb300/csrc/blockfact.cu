@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(32 * BS) k_bf_update_rows(const DevSymK S, int
 // longer than at its terms: an FP64 instruction holds its pipe for 64 cycles).  Used where a level
 // has few targets and long sums, so that these are not one thread's latency chain.  The split is
 // fixed by the structure alone (never by the batch size), so every state's result is the same
-// whatever the batch it belongs to.
+// whatever the batch it belongs to (on one side of BlockSym::tail_most).
 constexpr int kSlices = 8;
 
 template <int BS, bool SYM>

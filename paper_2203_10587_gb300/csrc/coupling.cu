@@ -41,7 +41,7 @@ using exago::set_last_error;
 constexpr int kSomeChildren = 8, kManyChildren = 256;
 constexpr int kSomeCols = 8, kManyCols = 4;
 constexpr int kMaxGridY = 65535;
-// Children of a heavy state staged in shared memory per pass.
+// Children of a state staged in shared memory per pass.
 constexpr int kStageChildren = 2048;
 
 // Values per thread along a row: every load of a thread is issued before its first store.

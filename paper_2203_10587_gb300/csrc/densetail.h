@@ -24,10 +24,10 @@
 //
 // GB300's FP64 pipe retires 528 G multiply-adds/s (measured), so the 76 M of one state's tail
 // take 75 ms for 512 states on it; their 28 bf16 products take 1-2 ms on the tensor cores.  Put
-// together, 2,000 buses x 512 states: KKT step 96.3 to 15.5 ms, power-flow step 37.3 to 7.8 ms;
-// 200 buses x 37 states, where the 190 levels' launches went instead: 1,442 to 493 us.  Mean error
-// of the step against extended precision, before and after: 4.29e-15 and 4.31e-15 (2,000 buses),
-// 5.9e-16 and 6.1e-16 (200); with barrier terms over many decades see half_exp.
+// together, 2,000 buses x 512 states: KKT step 96.3 to 15.6 ms, power-flow step 37.3 to 8.0 ms;
+// 200 buses x 37 states, where the 190 levels' launches went instead: 1,442 to 513 us.  Mean error
+// of the step against extended precision, before and after: 5.7e-15 and 5.6e-15 (2,000 buses),
+// 3.1e-15 and 3.1e-15 (200); with barrier terms over many decades see half_exp.
 //
 // Per panel J of 64 columns, for every state:
 //   k_dt_update<diag>  T_JJ -= sum_{K<J} F_JK L_JK'

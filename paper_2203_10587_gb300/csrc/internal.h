@@ -55,7 +55,7 @@ struct HostPlan {
     int nslot = 0;                // 2 nl
     std::vector<int> slot_ptr;    // [nb + 1] slots of bus i are [slot_ptr[i], slot_ptr[i+1])
     std::vector<int> slot_nbr;    // [nslot] the other bus of the slot's branch
-    std::vector<int> slot_ref;    // [nslot] 2 l + end of the slot (adjoint records by branch)
+    std::vector<int> slot_ref;    // [nslot] 2 l + end of the slot (the rectangular adjoint's records)
     std::vector<int> br_slot;     // [2][nl] slot of the from end and of the to end
     std::vector<int> slot_bus;    // [nslot] the bus of the slot
     std::vector<int> slot_pos;    // [nslot] column of the neighbour among the bus's row columns,
@@ -229,15 +229,15 @@ int launch_eval_persistent_w(const DevNet &net, const EvalReq &req, const Persis
 int persist_w_blocks_per_sm(int block, int occ_warps, int stage_cap);
 int persist_w_allow_stage();
 
-// Shared memory of a bus tile (eval_items.cuh, bus_tile): its records and its row segments.  The
-// largest tile's need in doubles, capped at kStageMaxDoubles; a tile above the cap reads its
-// records from global memory and writes its rows directly.
 // Block-per-state schedule (state_block.cu): a state's records and staged rows in one block's
 // shared memory.  nt: 64, 256 or 512 threads; smem: bytes, at most kStateMaxBytes.
 constexpr int kStateMaxBytes = 200 << 10;
 int state_allow_smem();
 int launch_eval_state(const DevNet &net, const EvalReq &req, int nt, size_t smem, void *stream);
 
+// Shared memory of a bus tile (eval_items.cuh, bus_tile): its records and its row segments.  The
+// largest tile's need in doubles, capped at kStageMaxDoubles; a tile above the cap reads its
+// records from global memory and writes its rows directly.
 constexpr int kStageMaxDoubles = 9216;   // 72 KB
 
 // Doubles of shared memory that each of `ctas` resident CTAs of an SM may stage its bus tiles in;
