@@ -40,6 +40,7 @@ using exago::set_last_error;
 // 256 / that rows of threads for its children (8 batched loads a thread cover 256 children with 32 rows).
 constexpr int kSomeChildren = 8, kManyChildren = 256;
 constexpr int kSomeCols = 8, kManyCols = 4;
+constexpr int kWaveBlocks = 152 * 8;   // such blocks resident at once
 constexpr int kMaxGridY = 65535;
 // Children of a state staged in shared memory per pass.
 constexpr int kStageChildren = 2048;
@@ -120,22 +121,28 @@ __device__ __forceinline__ void sum_children(const JtvArgs &A, int s, int g, int
 // lblocks blocks of kRowSpan generators each: the state's own row minus its children's, in ascending order.
 // A 512-state star (many): 8 children a thread in one batch of loads; with 8 generators x 32 rows they
 // were two, in a launch of its own (15.6 us the two launches).  With a dozen children a state the narrow
-// blocks are twice as many for nothing: 900 buses x 4,096 states 55 us with 4 generators a block, 30 with 8.
+// blocks are twice as many for nothing: 900 buses x 4,096 states 55 us with 4 generators a block, 30 with 8;
+// so are they where the wide ones fill the chip (a 512-state star of 17,500 generators 65 us, 54 wide).
+// WIDE = false: light states alone, without the others' shared memory.
+template <bool WIDE>
 __global__ void __launch_bounds__(256, 8) k_coupling_jtv(const JtvArgs A) {
-    __shared__ int kids[kStageChildren];
-    __shared__ double part[256 + 256 / kManyCols];
     const int tid = threadIdx.x, ng = A.ng;
-    const unsigned many_blocks = A.nmany * A.mblocks, some_blocks = A.nsome * A.sblocks;   // a grid holds all
-    if (blockIdx.x < many_blocks) {
-        sum_children<kManyCols>(A, __ldg(A.many + blockIdx.x / A.mblocks), blockIdx.x % A.mblocks, kids, part);
-        return;
+    unsigned blk = blockIdx.x;   // a grid holds all
+    if (WIDE) {
+        __shared__ int kids[kStageChildren];
+        __shared__ double part[256 + 256 / kManyCols];
+        const unsigned many_blocks = A.nmany * A.mblocks, some_blocks = A.nsome * A.sblocks;
+        if (blk < many_blocks) {
+            sum_children<kManyCols>(A, __ldg(A.many + blk / A.mblocks), blk % A.mblocks, kids, part);
+            return;
+        }
+        blk -= many_blocks;
+        if (blk < some_blocks) {
+            sum_children<kSomeCols>(A, __ldg(A.some + blk / A.sblocks), blk % A.sblocks, kids, part);
+            return;
+        }
+        blk -= some_blocks;
     }
-    if (blockIdx.x < many_blocks + some_blocks) {
-        const unsigned q = blockIdx.x - many_blocks;
-        sum_children<kSomeCols>(A, __ldg(A.some + q / A.sblocks), q % A.sblocks, kids, part);
-        return;
-    }
-    const unsigned blk = blockIdx.x - many_blocks - some_blocks;
     const int s = __ldg(A.light + blk / A.lblocks);
     const bool own = __ldg(A.parent + s) >= 0;
     const int c0 = __ldg(A.cptr + s), c1 = __ldg(A.cptr + s + 1);
@@ -267,7 +274,7 @@ exago_status exago_coupling_create(exago_net_t net, int B, const int *parent,
         p += c->child_idx.size();
         c->d_light = p;
         p += c->light.size();
-        c->d_some = p;
+        c->d_some = p;   // those with many follow
         p += c->some.size();
         c->d_many = p;
     }
@@ -343,17 +350,24 @@ exago_status exago_eval_coupling_jtv(exago_coupling_t c, const double *nu, doubl
     if (!nu || !out) return set_last_error(EXAGO_EINVAL, "nu or out is NULL");
     if (ldo < c->ng) return set_last_error(EXAGO_EINVAL, "ldo < ng");
     cudaStream_t s = (cudaStream_t)stream;
-    const int nlight = (int)c->light.size(), nsome = (int)c->some.size(), nmany = (int)c->many.size();
-    // states of one launch, so that its blocks fit the grid (2^31 - 1)
+    const int nlight = (int)c->light.size();
+    int nsome = (int)c->some.size(), nmany = (int)c->many.size();
     const int mb = (c->ng + kManyCols - 1) / kManyCols, sb = (c->ng + kSomeCols - 1) / kSomeCols;
     const int lb = (int)row_blocks(c->ng);
+    if ((int64_t)nmany * sb >= kWaveBlocks) {   // the wider blocks fill the chip: all in those
+        nsome += nmany;
+        nmany = 0;
+    }
+    // states of one launch, so that its blocks fit the grid (2^31 - 1)
     auto most = [](int blocks) { return std::max(1, (1 << 29) / blocks); };
     for (int m0 = 0, s0 = 0, l0 = 0; m0 < nmany || s0 < nsome || l0 < nlight;) {
         const int nm = std::min(most(mb), nmany - m0), ns = std::min(most(sb), nsome - s0);
         const int nl = std::min(most(lb), nlight - l0);
         const JtvArgs A{c->d_light + l0, c->d_some + s0, c->d_many + m0, c->d_parent, c->d_child_ptr,
                         c->d_child_idx, ns, nm, sb, mb, lb, c->ng, accumulate ? 1 : 0, nu, out, ldo};
-        k_coupling_jtv<<<(unsigned)(nm * mb + ns * sb + nl * lb), 256, 0, s>>>(A);
+        const unsigned blocks = nm * mb + ns * sb + nl * lb;
+        if (nm + ns > 0) k_coupling_jtv<true><<<blocks, 256, 0, s>>>(A);
+        else k_coupling_jtv<false><<<blocks, 256, 0, s>>>(A);
         m0 += nm;
         s0 += ns;
         l0 += nl;

@@ -21,10 +21,12 @@ def families(B, size):
     return p.astype(np.int32)
 
 
-@pytest.mark.parametrize("size", [9, 10, 12, 33, 65, 257, 258, 600])
-def test_families(ex, size):  # noqa: F811
+# the last: enough generators for blocks of 8 to fill the chip, whatever the children
+@pytest.mark.parametrize("size,ng", [(9, 23), (10, 23), (12, 23), (33, 23), (65, 23), (257, 23), (258, 23),
+                                     (600, 23), (300, 9801)])
+def test_families(ex, size, ng):  # noqa: F811
     import torch
-    g = synth.make_grid(3, 60, 90, 23)
+    g = synth.make_grid(3, max(60, ng), max(90, ng + 40), ng)
     net = ex.Net(g)
     B = 2 * size + 5   # two whole families, a rest, and one state with no family at all
     parent = families(B, size)
