@@ -602,12 +602,12 @@ exago_status exago_serve_drive(exago_server_t server, const exago_serve_client *
  * variables are eliminated first (they create no fill), then the remaining 4 x 4 block per bus
  * (Va, Vm, lamP, lamQ) is factored by a batched block L D L' without pivoting on a minimum-degree
  * order of the bus graph computed once by exago_kkt_create (the last columns, where the factor is
- * nearly full, as one dense matrix per state, with the same pivots in the same order; small grids
- * in batches too large for that to pay, a number of states that the grid decides, as all others.  A
- * state's result does not depend on the rest of its batch, nor on the batch's size on either side of
- * that number).  K must be factorable without
- * pivoting: it is whenever W + diag(dx) is positive definite and dc > 0 (a quasi-definite K;
- * interior-point methods regularise to that), and dx of every Qg must be nonzero.
+ * nearly full, as one dense matrix per state, with the same pivots in the same order; on small grids
+ * only in batches up to a number of states that the grid decides, beyond which that does not pay.
+ * A state's result depends neither on the rest of its batch nor on the batch's size on either side
+ * of that number).  K must be factorable without pivoting: it is whenever W + diag(dx) is positive
+ * definite and dc > 0 (a quasi-definite K; interior-point methods regularise to that), and dx of
+ * every Qg must be nonzero.
  *   exago_kkt_create      symbolic analysis on the host (ordering, factor structure, update
  *                         lists, levels) and upload.  On a net made by exago_net_plan it does the
  *                         analysis alone (info and order answer; solve returns ESTATE).  The
@@ -620,7 +620,8 @@ exago_status exago_serve_drive(exago_server_t server, const exago_serve_client *
  *   exago_kkt_workspace_size  scratch bytes for B states (two factor arrays of 16 x 8 B x B per
  *                         factor block, one without the dense last columns, whose panels and
  *                         split operands, up to 8 GB of them, come beside them; the reduced vectors
- *                         and counters): 2,000 buses x 512 states 8.3 GB.  Enough for every smaller batch too.
+ *                         and counters): 2,000 buses x 512 states 8.3 GB.  It is enough for every
+ *                         smaller batch too.
  *   exago_kkt_solve       DEVICE pointers, row-major per state: jval [B][nnzJ], hval [B][nnzH],
  *                         dx [B][n], dc [B][m] (> 0), rhs [B][n + m]; sol [B][n + m] receives
  *                         [dx; dlam].  inertia [B][2] (or NULL) receives the number of negative
@@ -630,9 +631,9 @@ exago_status exago_serve_drive(exago_server_t server, const exago_serve_client *
  *                         bytes, 256-byte aligned, or NULL for the handle's own (grown on demand;
  *                         a growth synchronises the device; calls using it must be ordered).
  *                         A smaller one is taken if it holds two whole factor arrays, the vectors
- *                         and counters, each rounded up to 256 bytes, and so is the handle's own
- *                         where the device has no room for more: the last columns are then factored as the
- *                         others are, which takes longer and rounds differently.
+ *                         and counters, each rounded up to 256 bytes, and the handle's own is of
+ *                         that size where the device has no room for more: the last columns are then
+ *                         factored as the others are, which takes longer and rounds differently.
  *                         Asynchronous on `stream`.  EINVAL for null arguments or B too large.
  */
 typedef struct exago_kkt *exago_kkt_t;
